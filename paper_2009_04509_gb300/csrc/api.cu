@@ -193,28 +193,26 @@ emtk_status run_network(emtk_ctx *c, const void *patches, const HitDesc *desc, i
                         const float *src32, cudaStream_t s) {
     if (n <= 0) return EMTK_OK;
     const int n_pad = n_pad_of(n);
-    const int max_splits = (int)std::max<int64_t>(1, kPartialCap / ((int64_t)n_pad * kN1));
+    const int max_rows = (int)std::max<int64_t>(1, kPartialCap / ((int64_t)n_pad * kN1));
     cudaError_t e;
-    int splits = 0, G = 0;
-    int *tile_done = nullptr;
-    if (tensor_precision(c->opt.precision)) {
-        // one persistent CTA per SM (stream-K), fewer if the partial rows would not fit
-        G = c->sm_count;
-        while (G > 1 && streamk_partial_rows(n, G) > max_splits) G /= 2;
-        // the head of a large launch takes each tile as soon as its partial rows are stored
-        if (head_counts_tiles(n, G)) tile_done = c->ws.tile_done;
+    const bool tc = tensor_precision(c->opt.precision);
+    const int upt = tc ? kQuads : kPos / 2;
+    // one persistent CTA per SM (stream-K), fewer if the partial rows would not fit
+    int G = c->sm_count;
+    while (G > 1 && streamk_partial_rows(n, G, upt) > max_rows) G /= 2;
+    // the head of a large launch takes each tile as soon as its partial rows are stored
+    // (the tensor-core kernels count them; no kernel of the fp32 path waits on another)
+    int *tile_done = tc && head_counts_tiles(n, G, upt) ? c->ws.tile_done : nullptr;
+    {
         Prof prof(c, EMTK_KERNEL_NETWORK, s);
-        e = launch_cnn_tc(c->w, patches, desc, tc_mode(c->opt.precision), n, G, c->ws.partials, n_pad,
-                          c->ws.status, c->opt.wait_timeout_ns, c->opt.debug_stall, tile_done, src32, s);
-    } else {
-        splits = choose_splits_fp32(n, c->sm_count, max_splits);
-        Prof prof(c, EMTK_KERNEL_NETWORK, s);
-        e = launch_cnn_fp32(c->w, static_cast<const float *>(patches), n, splits, c->ws.partials, n_pad, s);
+        e = tc ? launch_cnn_tc(c->w, patches, desc, tc_mode(c->opt.precision), n, G, c->ws.partials, n_pad,
+                               c->ws.status, c->opt.wait_timeout_ns, c->opt.debug_stall, tile_done, src32, s)
+               : launch_cnn_fp32(c->w, static_cast<const float *>(patches), n, G, c->ws.partials, n_pad, s);
     }
     if (e != cudaSuccess) return cuda_status(e);
     {
         Prof prof(c, EMTK_KERNEL_HEAD, s);
-        e = launch_head(c->w, c->ws.partials, splits, G, n_pad, n, out_rows, c->opt.debug_logits, tile_done,
+        e = launch_head(c->w, c->ws.partials, G, upt, n_pad, n, out_rows, c->opt.debug_logits, tile_done,
                         c->ws.status, c->opt.wait_timeout_ns, s);
     }
     count_launch(c, n);
@@ -491,8 +489,6 @@ emtk_status emtk_create(const emtk_weights *w, const emtk_options *opt, int devi
     DeviceWeights &d = c->w;
     if (e == cudaSuccess) e = upload(&d.conv_w, w->conv_w, (size_t)kK * kK * kF);
     if (e == cudaSuccess) e = upload(&d.conv_b, w->conv_b, kF);
-    std::copy(w->conv_w, w->conv_w + kK * kK * kF, d.conv_w_host);
-    std::copy(w->conv_b, w->conv_b + kF, d.conv_b_host);
     if (e == cudaSuccess) e = upload(&d.fc1_b, w->fc1_b, kN1);
     if (e == cudaSuccess) e = upload(&d.fc2_w, w->fc2_w, (size_t)kN1 * kN2);
     if (e == cudaSuccess) e = upload(&d.fc2_b, w->fc2_b, kN2);

@@ -1,166 +1,290 @@
 // fp32 network path on CUDA cores (EMTK_FP32): conv 5x5x48 + ReLU fused
-// with dense-1 (Sec. 2.2), split over the dense-1 input dimension (the conv
-// positions) into `splits` segments.
+// with dense-1 (Sec. 2.2).
 //
-// Block = 128 hits x one segment of conv positions, 256 threads.  Per
-// position the block
-//   - computes the 128 x 48 conv activations (thread: one hit, 24 filters;
-//     each warp one half of the filters) from a 5-row band of the hits'
-//     patches held in shared memory (rows kept by row % 5, one new row per
-//     output row), transposed into act[48][128].  The conv weights are a
-//     launch parameter, so the FMAs read them from the constant bank: one
-//     shared-memory load per tap and thread;
-//   - multiplies them into the dense-1 sums with the position's 48 x 128
-//     weights, which cp.async brought into one of two shared buffers while
-//     the previous position was computed: thread (hit group g, output group
-//     o) accumulates hits 8g..8g+7 x outputs 4o..4o+3 and 64+4o..64+4o+3 in
-//     64 registers (the split keeps the weight loads free of bank
-//     conflicts), 16 FMAs per shared-memory load.
-// Segment partial sums go to partials[segment][hit][128]; the head kernel
-// adds them in segment order, so results are deterministic.
+// Work units are (tile of 128 hits, pair of conv positions (x, x + 1), x even):
+// 968 per tile.  One persistent CTA per SM takes a contiguous range of units
+// (stream-K), across tile boundaries, so every SM gets the same work (+-1 pair)
+// whatever the hit count; a grid of whole K splits left the last of 2 to 5
+// waves mostly empty (628 CTAs on 152 SMs for 20,000 hits).  256 threads, a conv
+// warp and a dense-1 warp on each SM sub-partition, joined by a ring of two
+// shared-memory slots (one pair each: its 96 x 128 dense-1 weights and its
+// 96 x 128 activations):
+//   conv warps     bring the pair's dense-1 weights in (cp.async) and compute
+//                  its activations: the 5 x 8 window of a quad of positions is
+//                  staged in shared memory, a thread takes two hits and 24
+//                  filters, one window row per loop iteration;
+//   dense-1 warps  16 hits x 8 outputs per thread in 64 packed pairs of hits,
+//                  the next input's 6 shared-memory loads in flight under the
+//                  current one's 64 FMAs.
+// Both use the packed FMA (two IEEE fp32 FMAs per instruction): the FMA pipe
+// runs 128 FMAs per cycle and SM either way, but the packed form leaves half
+// the issue slots to loads, to the copies that put a scalar into both halves of
+// a pair, and to the other warp.  Both loops are short on purpose: straight-line
+// code that does not fit the instruction cache ran at a quarter of its rate (a
+// fully unrolled conv took 6,000 cycles per position for 1,200 FMAs).
+//
+// What bounds it: the FMA pipe.  A position is 7,344 pipe cycles; it takes about
+// 9,300 (20,096 hits: 9.6 ms, 60 TFLOP/s, 0.75 of the derived peak; the kernel
+// before this one 13.5 ms).  Operands that are all 64-bit pairs straight from
+// shared memory (each activation stored twice, no copies) ran at 42 TFLOP/s, an
+// 8 x 8 register tile on twice the warps at 59, scalar FMAs at 53.
+//
+// The dense-1 sums restart every `seg` positions of a tile and are added to
+// the CTA's partial row of the tile with one fp32 add per segment, in order
+// (deterministic; shorter chains of sums round less).  The head kernel adds
+// the partial rows of the CTAs that shared a tile, in CTA order.
 #include "emtk_internal.h"
 
 namespace emtk {
 namespace {
 
-constexpr int kHT = 128;      // hits per block
-constexpr int kThreads = 256;
-constexpr int kBandStride = kPatch + 1;  // 49: conflict-free per-hit reads
-constexpr int kW1Pos = kF * kN1;         // 6144 weights of one position (24 KB)
-// shared memory: band[5][128][49], w1[2][48][128], act[48][128]
-constexpr int kSmemFloats = kK * kHT * kBandStride + 2 * kW1Pos + kF * kHT;
-constexpr int kSmemBytes = kSmemFloats * 4;
+constexpr int kHT = 128;          // hits per tile
+constexpr int kRole = 128;        // threads of each role
+constexpr int kThreads = 2 * kRole;
+constexpr int kPairs = kPos / 2;   // units per tile: pairs of conv positions (x, x + 1), x even
+constexpr int kSlots = 4;          // ring slots (positions)
+constexpr int kW1Pos = kF * kN1;   // 6144 weights of one position (24 KB)
+constexpr int kActPos = kF * kHT;  // 6144 activations of one position
+constexpr int kWinHalf = kK * kHT * 4;      // 5 rows x 128 hits x 4 columns of a quad's window
+constexpr int kConvF = kK * kK * kF + kF;   // conv weights [25][48], then the bias [48]
+constexpr int kSmemBytes = (kSlots * (kW1Pos + kActPos) + 2 * kWinHalf + kConvF) * 4;
 static_assert(kSmemBytes <= 232448, "shared memory budget");
-static_assert(kW1Pos % (4 * kThreads) == 0 && kHT % 32 == 0 && kThreads == 2 * kHT && kThreads / 16 * 8 == kHT,
-              "thread layout: two conv filter halves of kHT hits; 16 threads per 8 hits in dense-1");
+static_assert((kSlots & (kSlots - 1)) == 0, "slot index by mask");
+static_assert(kW1Pos % (4 * kRole) == 0 && kQ % 4 == 0, "whole vectors per thread; quads do not straddle rows");
 
 __device__ __forceinline__ void cp_async16(float *smem_dst, const float *gmem_src) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// The 48 x 128 dense-1 weights of position p into dst (each thread 6 x 16 bytes).
-__device__ __forceinline__ void load_w1(float *dst, const float *__restrict__ fc1_w, int p, int tid) {
+// Named barriers of the ring: pair b (two slots) is full at kBarFull + b (conv
+// warps arrive, dense-1 warps wait) and free at kBarFree + b (the other way
+// round); kBarConv joins the conv warps.
+constexpr int kBarFull = 1, kBarFree = 3, kBarConv = 5;
+__device__ __forceinline__ void bar_wait(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kThreads) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kThreads) : "memory");
+}
+__device__ __forceinline__ void bar_conv() { asm volatile("bar.sync %0, %1;" ::"n"(kBarConv), "n"(kRole) : "memory"); }
+
+// The 48 x 128 dense-1 weights of position p into dst: thread t's share, copied
+// asynchronously.
+__device__ __forceinline__ void load_w1(float *dst, const float *__restrict__ fc1_w, int p, int t) {
     const float *src = fc1_w + (int64_t)p * kW1Pos;
 #pragma unroll
-    for (int k = 0; k < kW1Pos / 4 / kThreads; ++k) {
-        const int i = (tid + k * kThreads) * 4;
-        cp_async16(dst + i, src + i);
-    }
+    for (int k = 0; k < kW1Pos / 4 / kRole; ++k) cp_async16(dst + (t + k * kRole) * 4, src + (t + k * kRole) * 4);
 }
 
-// Patch row `prow` of the block's 128 hits into band slot prow % 5 (zero past n).
-__device__ __forceinline__ void load_band_row(float *band, const float *__restrict__ patches, int n, int hit0, int prow,
-                                              int tid) {
-    float *slot = band + (prow % kK) * kHT * kBandStride;
-    for (int i = tid; i < kHT * kPatch / 4; i += kThreads) {
-        const int h = i / (kPatch / 4), c4 = i - h * (kPatch / 4);
-        const int gh = hit0 + h;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (gh < n) v = __ldg(reinterpret_cast<const float4 *>(patches + (int64_t)gh * kPatchElems + prow * kPatch) + c4);
-        float *d = slot + h * kBandStride + 4 * c4;
-        d[0] = v.x;
-        d[1] = v.y;
-        d[2] = v.z;
-        d[3] = v.w;
+// Conv + ReLU of positions x, x + 1 (window columns C0 .. C0 + 5 of the staged
+// quad) for two hits, 32 apart, and 24 filters, into the pair's activations.  One
+// window row's 5 taps per iteration (a loop that stays in the instruction
+// cache): per tap, 12 packed filter pairs x 2 positions x 2 hits on 6 weight
+// loads, which every lane reads at once.
+template <int C0>
+__device__ __forceinline__ void conv_pair(const float *win, const float *cw, float *act) {
+    float2 s[2][2][12];  // [hit][position][filter pair]
+    const float2 *bias = reinterpret_cast<const float2 *>(cw + kK * kK * kF);
+#pragma unroll
+    for (int f = 0; f < 12; ++f) s[0][0][f] = s[0][1][f] = s[1][0][f] = s[1][1][f] = bias[f];
+#pragma unroll 1
+    for (int r = 0; r < kK; ++r, cw += kK * kF, win += kHT * 4) {
+        float px[2][8];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 lo = *reinterpret_cast<const float4 *>(win + h * 32 * 4);
+            const float4 hi = *reinterpret_cast<const float4 *>(win + h * 32 * 4 + kWinHalf);
+            px[h][0] = lo.x, px[h][1] = lo.y, px[h][2] = lo.z, px[h][3] = lo.w;
+            px[h][4] = hi.x, px[h][5] = hi.y, px[h][6] = hi.z, px[h][7] = hi.w;
+        }
+#pragma unroll
+        for (int j = 0; j < kK; ++j)
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const float4 w = *reinterpret_cast<const float4 *>(cw + j * kF + 4 * q);
+                const float2 wl = make_float2(w.x, w.y), wh = make_float2(w.z, w.w);
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        const float2 v = make_float2(px[h][C0 + j + x], px[h][C0 + j + x]);
+                        s[h][x][2 * q] = __ffma2_rn(v, wl, s[h][x][2 * q]);
+                        s[h][x][2 * q + 1] = __ffma2_rn(v, wh, s[h][x][2 * q + 1]);
+                    }
+            }
     }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int f = 0; f < 12; ++f) {
+                float *d = act + x * kActPos + 2 * f * kHT + 32 * h;
+                d[0] = fmaxf(s[h][x][f].x, 0.0f);
+                d[kHT] = fmaxf(s[h][x][f].y, 0.0f);
+            }
 }
 
-// The conv weights [25][48] and bias [48], passed by value.
-struct ConvParams {
-    float w[kK * kK * kF];
-    float b[kF];
+// One input's operands of a dense-1 thread: 16 hits (4 x 4, 32 apart) and 8
+// outputs (2 x 4, 64 apart).
+struct Frag {
+    float4 a[4], b[2];
+    __device__ __forceinline__ void load(const float *act, const float *w1, int c) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a[j] = *reinterpret_cast<const float4 *>(act + c * kHT + 32 * j);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) b[j] = *reinterpret_cast<const float4 *>(w1 + c * kN1 + 64 * j);
+    }
 };
 
-// Conv + ReLU of hit `hit` at position (y, x), filters F0 .. F0+23, into act.
-template <int F0>
-__device__ __forceinline__ void conv_half(const ConvParams &cp, const float *band, int y, int x, int hit, float *act) {
-    float s[24];
+// acc[q][o] (pair of hits q, output o) += the pair's activations x the weight of o.
+__device__ __forceinline__ void fma_frag(const Frag &f, float2 (&acc)[8][8]) {
+    const float b[8] = {f.b[0].x, f.b[0].y, f.b[0].z, f.b[0].w, f.b[1].x, f.b[1].y, f.b[1].z, f.b[1].w};
 #pragma unroll
-    for (int f = 0; f < 24; ++f) s[f] = cp.b[F0 + f];
+    for (int q = 0; q < 8; ++q) {
+        const float4 v = f.a[q >> 1];
+        const float2 a = q & 1 ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
 #pragma unroll
-    for (int i = 0; i < kK; ++i) {
-        const float *row = band + ((y + i) % kK) * kHT * kBandStride + hit * kBandStride + x;
-#pragma unroll
-        for (int j = 0; j < kK; ++j) {
-            const float v = row[j];
-#pragma unroll
-            for (int f = 0; f < 24; ++f) s[f] = fmaf(v, cp.w[(i * kK + j) * kF + F0 + f], s[f]);
-        }
+        for (int o = 0; o < 8; ++o) acc[q][o] = __ffma2_rn(a, make_float2(b[o], b[o]), acc[q][o]);
     }
-#pragma unroll
-    for (int f = 0; f < 24; ++f) act[(F0 + f) * kHT + hit] = fmaxf(s[f], 0.0f);
 }
 
-__global__ void __launch_bounds__(kThreads, 1) cnn_fp32_kernel(const float *__restrict__ patches, int n,
-                                                               const __grid_constant__ ConvParams cp,
-                                                               const float *__restrict__ fc1_w, int splits,
-                                                               float *__restrict__ partials, int n_pad) {
+// units = tiles * kPairs pairs in all; seg: positions per dense-1 segment.
+__global__ void __launch_bounds__(kThreads, 1)
+    cnn_fp32_kernel(const float *__restrict__ patches, int n, const float *__restrict__ conv_w,
+                    const float *__restrict__ conv_b, const float *__restrict__ fc1_w, long long units,
+                    float *__restrict__ partials, int n_pad, int seg) {
     extern __shared__ float4 smem_f4[];
-    float *band = reinterpret_cast<float *>(smem_f4);  // [5][128][49]
-    float *w1 = band + kK * kHT * kBandStride;          // [2][48][128]
-    float *act = w1 + 2 * kW1Pos;                       // [48][128]
+    float *w1 = reinterpret_cast<float *>(smem_f4);  // [kSlots][48][128]
+    float *act = w1 + kSlots * kW1Pos;               // [kSlots][48][128]
+    float *win = act + kSlots * kActPos;             // [2][5][128][4]
+    float *cw = win + 2 * kWinHalf;                  // [25][48], [48]
+    const int cta = blockIdx.x, G = gridDim.x;
+    const int64_t u0 = unit_begin(cta, units, G), u1 = unit_begin(cta + 1, units, G);
+    const int np = 2 * (int)(u1 - u0);  // positions, in order, across tile boundaries
+    int64_t tile = u0 / kPairs;
+    int p = 2 * (int)(u0 - tile * kPairs);
+    pdl_trigger();  // the head may be scheduled as SMs free up; it waits for this kernel
 
-    const int tid = threadIdx.x;
-    const int hit0 = blockIdx.x * kHT;
-    const int seg = blockIdx.y;
-    const int p_begin = (int)((int64_t)seg * kPos / splits);
-    const int p_end = (int)((int64_t)(seg + 1) * kPos / splits);
-
-    const int g = tid >> 4, o = tid & 15;  // dense-1: hits 8g.., outputs 4o.. and 64+4o..
-    const int ch = tid & (kHT - 1);        // conv: hit ch, filter half tid / 128 (one per warp)
-    float acc[8][8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
-
-    if (p_begin < p_end) load_w1(w1, fc1_w, p_begin, tid);
-    cp_async_commit();
-    int band_y = -1;
-    for (int p = p_begin; p < p_end; ++p) {
-        const int y = p / kQ, x = p - y * kQ;
-        // the next position's weights into the other buffer (free since the last barrier)
-        if (p + 1 < p_end) load_w1(w1 + ((p + 1 - p_begin) & 1) * kW1Pos, fc1_w, p + 1, tid);
-        cp_async_commit();
-        if (y != band_y) {  // rows y..y+4: all five at the segment's start, then the one new row
-            for (int r = band_y < 0 ? y : y + kK - 1; r < y + kK; ++r) load_band_row(band, patches, n, hit0, r, tid);
-            band_y = y;
-            __syncthreads();
+    if (threadIdx.x >= kRole) {
+        // ================================================= conv + weights
+        const int t = threadIdx.x - kRole;
+        for (int i = t; i < kConvF; i += kRole) cw[i] = i < kK * kK * kF ? conv_w[i] : conv_b[i - kK * kK * kF];
+        if (np > 0) {
+            load_w1(w1, fc1_w, p, t);
+            load_w1(w1 + kW1Pos, fc1_w, p + 1, t);
         }
-        // conv + ReLU, transposed into act
-        if (tid < kHT)
-            conv_half<0>(cp, band, y, x, ch, act);
-        else
-            conv_half<24>(cp, band, y, x, ch, act);
-        cp_async_wait_prev();  // this position's weights have landed
-        __syncthreads();
-        // dense-1: 8 hits x 8 outputs per thread
-        const float *wp = w1 + ((p - p_begin) & 1) * kW1Pos;
-#pragma unroll 4
-        for (int c = 0; c < kF; ++c) {
-            const float4 a0 = *reinterpret_cast<const float4 *>(act + c * kHT + 8 * g);
-            const float4 a1 = *reinterpret_cast<const float4 *>(act + c * kHT + 8 * g + 4);
-            const float4 b0 = *reinterpret_cast<const float4 *>(wp + c * kN1 + 4 * o);
-            const float4 b1 = *reinterpret_cast<const float4 *>(wp + c * kN1 + 64 + 4 * o);
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        pdl_wait();  // the patches come from the kernel before
+        const int hit_c = 64 * ((t >> 5) & 1) + (t & 31), f_c = 24 * (t >> 6);  // this thread's conv: hits, filters
+        for (int i = 0; i < np; i += 2) {
+            // the pair of position p: window rows y .. y+4, columns x0 .. x0+7 of its quad
+            const int y = p / kQ, x = p - y * kQ, x0 = x & ~3;
+            if (i == 0 || x == x0) {  // a new quad: thread t stages hit t's window
+                const int64_t hit = tile * kHT + t;
+                const float4 *src = reinterpret_cast<const float4 *>(patches + hit * kPatchElems + y * kPatch + x0);
+                float4 a[kK], b[kK];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+                for (int r = 0; r < kK; ++r) {
+                    a[r] = hit < n ? __ldg(src + r * (kPatch / 4)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    b[r] = hit < n ? __ldg(src + r * (kPatch / 4) + 1) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                }
+                bar_conv();  // the last quad's window has been read (first: the conv weights are staged)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int r = 0; r < kK; ++r) {
+                    *reinterpret_cast<float4 *>(win + (r * kHT + t) * 4) = a[r];
+                    *reinterpret_cast<float4 *>(win + kWinHalf + (r * kHT + t) * 4) = b[r];
+                }
+                bar_conv();
+            }
+            // the pair's weights, in flight under its conv
+            const int s = i & (kSlots - 1), b = s >> 1;
+            if (i >= kSlots) bar_wait(kBarFree + b);
+            if (i > 0) {
+                load_w1(w1 + s * kW1Pos, fc1_w, p, t);
+                load_w1(w1 + (s + 1) * kW1Pos, fc1_w, p + 1, t);
+            }
+            if (x == x0)
+                conv_pair<0>(win + 4 * hit_c, cw + f_c, act + s * kActPos + f_c * kHT + hit_c);
+            else
+                conv_pair<2>(win + 4 * hit_c, cw + f_c, act + s * kActPos + f_c * kHT + hit_c);
+            cp_async_wait_all();  // this thread's share of the weights has landed
+            bar_arrive(kBarFull + b);
+            p += 2;
+            if (p == kPos) {
+                p = 0;
+                ++tile;
+            }
         }
-        __syncthreads();
+        return;
     }
+
+    // =========================================================== dense-1
+    // thread: hits 32 j + 4 hg .. +3 (j = 0..3), outputs 64 j + 4 og .. +3 (j = 0, 1).
+    // A 16-byte shared-memory load of a warp takes two passes instead of four when
+    // lanes l and l ^ 1, or lanes l and l ^ 2, share every address (2.1 against 4.0
+    // cycles): bit 0 of the lane moves only the hits, bit 1 only the outputs.
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int hg = 4 * (warp & 1) + ((lane & 1) | ((lane >> 1) & 2));
+    const int og = 8 * (warp >> 1) + (((lane >> 1) & 1) | ((lane >> 2) & 6));
+    float2 acc[8][8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int gh = hit0 + 8 * g + i;
-        if (gh < n) {
-            float *dst = partials + ((int64_t)seg * n_pad + gh) * kN1;
-            reinterpret_cast<float4 *>(dst + 4 * o)[0] = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-            reinterpret_cast<float4 *>(dst + 64 + 4 * o)[0] = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+    for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int o = 0; o < 8; ++o) acc[q][o] = make_float2(0.0f, 0.0f);
+    int64_t started = -1;  // tile whose partial row this CTA has begun
+    for (int i = 0; i < np; i += 2) {
+        const int s = i & (kSlots - 1), b = s >> 1;
+        bar_wait(kBarFull + b);
+        // a pair's 96 inputs: its two slots are contiguous
+        const float *a = act + s * kActPos + 4 * hg, *w = w1 + s * kW1Pos + 4 * og;
+        Frag f0, f1;
+        f0.load(a, w, 0);
+        // unconditional loads (the last one is a repeat): a conditional one costs a
+        // copy of the whole operand set per input
+#pragma unroll 1
+        for (int c = 0; c < 2 * kF; c += 2) {
+            f1.load(a, w, c + 1);
+            fma_frag(f0, acc);
+            f0.load(a, w, c + 2 < 2 * kF ? c + 2 : 0);
+            fma_frag(f1, acc);
+        }
+        if (i + kSlots < np) bar_arrive(kBarFree + b);
+        p += 2;
+        if (i == np - 2 || p == kPos || p % seg == 0) {  // the segment's sums onto the partial row
+            const int krow = cta - cta_of_unit(tile * kPairs, units, G);
+            const bool first = tile != started;
+            started = tile;
+            // rows past n lie in the padding of the tile and are never read.  Four hits at
+            // a time: their loads before their stores
+            float *row = partials + ((int64_t)krow * n_pad + tile * kHT + 4 * hg) * kN1 + 4 * og;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float4 *dst = reinterpret_cast<float4 *>(row + 32 * j * kN1);
+                float4 old[4][2];
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+#pragma unroll
+                    for (int k = 0; k < 2; ++k)
+                        old[h][k] = first ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : dst[(h * kN1 + 64 * k) / 4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        const float2 *v = acc[2 * j + (h >> 1)] + 4 * k;
+                        const float4 o = old[h][k];
+                        dst[(h * kN1 + 64 * k) / 4] =
+                            h & 1 ? make_float4(o.x + v[0].y, o.y + v[1].y, o.z + v[2].y, o.w + v[3].y)
+                                  : make_float4(o.x + v[0].x, o.y + v[1].x, o.z + v[2].x, o.w + v[3].x);
+                    }
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+#pragma unroll
+                for (int o = 0; o < 8; ++o) acc[q][o] = make_float2(0.0f, 0.0f);
+        }
+        if (p == kPos) {
+            p = 0;
+            ++tile;
         }
     }
 }
@@ -171,24 +295,14 @@ cudaError_t init_fp32_kernel_attrs() {
     return cudaFuncSetAttribute(cnn_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
 }
 
-// K splits: about four waves of one-block-per-SM work, at least 16 positions per split.
-int choose_splits_fp32(int n, int sm_count, int max_splits) {
-    const int blocks = (n + kHT - 1) / kHT;
-    int s = (4 * sm_count + blocks - 1) / blocks;
-    if (s > kPos / 16) s = kPos / 16;
-    if (s > max_splits) s = max_splits;
-    return s < 1 ? 1 : s;
-}
-
-cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *patches, int32_t n, int splits, float *partials,
+cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *patches, int32_t n, int G, float *partials,
                             int n_pad, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    ConvParams cp;
-    for (int i = 0; i < kK * kK * kF; ++i) cp.w[i] = w.conv_w_host[i];
-    for (int i = 0; i < kF; ++i) cp.b[i] = w.conv_b_host[i];
-    dim3 grid((n + kHT - 1) / kHT, splits);
-    cnn_fp32_kernel<<<grid, kThreads, kSmemBytes, s>>>(patches, n, cp, w.fc1_w, splits, partials, n_pad);
-    return cudaGetLastError();
+    const long long units = (long long)((n + kHT - 1) / kHT) * kPairs;
+    const int seg = units <= 88ll * G ? 16 : kQ;
+    const float *cw = w.conv_w, *cb = w.conv_b, *fw = w.fc1_w;
+    return launch_pdl(cnn_fp32_kernel, dim3(G), dim3(kThreads), kSmemBytes, s, patches, n, cw, cb, fw, units,
+                      partials, n_pad, seg);
 }
 
 }  // namespace emtk

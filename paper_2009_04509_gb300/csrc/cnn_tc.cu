@@ -806,14 +806,13 @@ cudaError_t prepare_tc_weights(DeviceWeights &w, const emtk_weights &hw, TcMode 
 
 // Partial-sum rows a stream-K launch over G CTAs needs: the largest number
 // of CTAs that share one tile.
-int streamk_partial_rows(int32_t n, int G) {
+int streamk_partial_rows(int32_t n, int G, int upt) {
     const int m_tiles = (n + 127) / 128;
-    const int64_t units = (int64_t)m_tiles * kW1Steps;
+    const int64_t units = (int64_t)m_tiles * upt;
     int rows = 1;
     for (int t = 0; t < m_tiles; ++t) {
-        const int a = cta_of_unit((int64_t)t * kW1Steps, units, G);
-        const int b = cta_of_unit((int64_t)t * kW1Steps + kW1Steps - 1, units, G);
-        rows = b - a + 1 > rows ? b - a + 1 : rows;
+        const int r = tile_partial_rows(t, units, G, upt);
+        rows = r > rows ? r : rows;
     }
     return rows;
 }

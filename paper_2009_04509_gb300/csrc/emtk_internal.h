@@ -25,17 +25,22 @@ constexpr int kNC = 3;
 constexpr int kPatchElems = kPatch * kPatch;         // 2304
 constexpr int kQuads = kPos / 4;                     // 484 quads of 4 conv positions
 
-// Stream-K split of the tensor-core network: the launch's work is the units
-// u = tile * kQuads + quad (tile = 128 hits); CTA c of G takes the contiguous
-// units [unit_begin(c), unit_begin(c + 1)).  A tile's dense-1 partial sums
-// come from CTAs cta_of_unit(first unit) .. cta_of_unit(last unit), written
-// to partial rows 0, 1, ... in that order.
+// Stream-K split of the network kernels: the launch's work is the units
+// u = tile * upt + i (tile = 128 hits; upt units per tile: kQuads quads of
+// conv positions on the tensor cores, kPos / 2 pairs in fp32); CTA c of G
+// takes the contiguous units [unit_begin(c), unit_begin(c + 1)).  A tile's
+// dense-1 partial sums come from CTAs cta_of_unit(first unit) ..
+// cta_of_unit(last unit), written to partial rows 0, 1, ... in that order.
 __host__ __device__ inline int64_t unit_begin(int c, int64_t units, int G) { return (int64_t)c * units / G; }
 __host__ __device__ inline int cta_of_unit(int64_t u, int64_t units, int G) {
     int c = (int)((u * G) / units);
     while (c > 0 && unit_begin(c, units, G) > u) --c;
     while (c + 1 < G && unit_begin(c + 1, units, G) <= u) ++c;
     return c;
+}
+
+__host__ __device__ inline int tile_partial_rows(int64_t tile, int64_t units, int G, int upt) {
+    return cta_of_unit(tile * upt + upt - 1, units, G) - cta_of_unit(tile * upt, units, G) + 1;
 }
 
 // Requests handled by one extraction launch (kernel-parameter table).
@@ -116,7 +121,7 @@ struct Workspace {
     void *patches = nullptr;     // [max_hits][48][48] in the precision's patch format
     HitDesc *hdesc = nullptr;    // [max_hits] window descriptors (tensor-core path)
     float **dest = nullptr;      // [max_hits] output row of each hit
-    float *partials = nullptr;   // [max_splits][max_hits_pad][128]
+    float *partials = nullptr;   // [rows][n_pad][128] of the running launch
     size_t partial_elems = 0;
     int *status = nullptr;       // device status word (bit 0: a network wait gave up, bit 1: a head wait)
     int *tile_done = nullptr;    // [max_hits / 128 + 1] per tile: epilogue warps whose partial rows are stored
@@ -140,10 +145,6 @@ struct DeviceWeights {
     float fc1_scale = 1.0f;        // dense-1 sums are scaled by this before the bias (EMTK_FP8: 1/(s_a s_w))
     float fc1_w_scale = 1.0f;      // EMTK_FP8 / EMTK_TF32: s_w, the power of two the weights were scaled by
     float act_mul = 1.0f;          // EMTK_TF32: s_a / (s_p s_c), applied to the ReLU'd conv sums
-    // host copy of the conv weights [25][48] and bias [48]: the fp32 kernel takes
-    // them as a launch parameter (constant bank)
-    float conv_w_host[kK * kK * kF] = {};
-    float conv_b_host[kF] = {};
 };
 
 // Operand formats of the tensor-core kernels: 16-bit (cnn_tc.cu, also with
@@ -197,7 +198,6 @@ struct emtk_ctx {
     std::vector<emtk_pending_event> pending;  // profile mode: launches not yet read back
     emtk_options opt{};
     int max_hits = 0;
-    int max_splits = 0;
     int sm_count = 0;
     emtk::DeviceWeights w;
     emtk::Workspace ws;
@@ -295,11 +295,12 @@ int64_t find_hits_chunks(const HfTable &t, int64_t nunits);
 cudaError_t launch_find_hits(const HfTable &t, int64_t nunits, void *scratch, int32_t *sums_cur, int32_t *sums_next,
                              int64_t cap, int32_t *totals, cudaStream_t s);
 
-// Network: dense-1 partial sums [splits][n_pad][128] from patches.
-cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *patches, int32_t n, int splits,
-                            float *partials, int n_pad, cudaStream_t s);
+// Network in fp32: dense-1 partial sums [rows][n_pad][128] from patches, stream-K
+// over G CTAs in pairs of positions (rows = streamk_partial_rows(n, G, kPos / 2)).
+cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *patches, int32_t n, int G, float *partials,
+                            int n_pad, cudaStream_t s);
 // Stream-K over G CTAs (one per SM); partials [rows][n_pad][128] with rows
-// = streamk_partial_rows(n, G).
+// = streamk_partial_rows(n, G, kQuads).
 // src: 16-bit patches [n][48][48] (desc == nullptr) or the haloed interval
 // images of the hits' planes, located through desc.
 // tile_done (or null): each epilogue warp adds 1 to tile_done[tile] once its
@@ -318,16 +319,15 @@ struct OutRows {
     float *rows;
     int stride;
 };
-int streamk_partial_rows(int32_t n, int G);
+int streamk_partial_rows(int32_t n, int G, int upt);
 // Sum of partials + bias + ReLU, dense-2, heads; hit h's scores where out_rows says.  Partial
-// rows: `splits` per hit (G == 0), or the stream-K contributors of the hit's
-// tile (G > 0).  With tile_done (stream-K launches for which
-// head_counts_tiles(n, G) holds), a tile's head starts once the tile's
-// counter is complete instead of after the whole network kernel, gives up
-// when bit 0 of *status is set or after timeout_ns (setting bit 1), and
-// sets the counter back to zero.
-bool head_counts_tiles(int32_t n, int G);
-cudaError_t launch_head(const DeviceWeights &w, const float *partials, int splits, int G, int n_pad,
+// rows: the stream-K contributors of the hit's tile (G CTAs, upt units per
+// tile).  With tile_done (launches for which head_counts_tiles(n, G, upt)
+// holds), a tile's head starts once the tile's counter is complete instead of
+// after the whole network kernel, gives up when bit 0 of *status is set or
+// after timeout_ns (setting bit 1), and sets the counter back to zero.
+bool head_counts_tiles(int32_t n, int G, int upt);
+cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, int upt, int n_pad,
                         int32_t n, OutRows out_rows, int debug_logits, int *tile_done, int *status,
                         int64_t timeout_ns, cudaStream_t s);
 
@@ -345,6 +345,5 @@ cudaError_t launch_cnn_split(const DeviceWeights &w, const void *src, const HitD
                              int *tile_done, cudaStream_t s);
 // EMTK_FP8 weight scale: the largest power of two s_w with max|W1| s_w <= 448.
 double fp8_weight_scale(const float *fc1_w, size_t n);
-int choose_splits_fp32(int n, int sm_count, int max_splits);
 
 }  // namespace emtk

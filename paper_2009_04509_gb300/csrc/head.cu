@@ -1,8 +1,8 @@
 // Network tail (Sec. 2.2), fp32: sum of the dense-1 partial-sum rows in row
 // order, times the dense-1 scale s1 (1, or the inverse of the operand scales
 // of the e4m3 path), + bias + ReLU, dense 128->32 + ReLU, the 3-way softmax
-// head (track, em, none) and the Michel sigmoid head.  The rows of a hit are
-// the K-splits of the fp32 path, or the stream-K CTAs that shared its tile.
+// head (track, em, none) and the Michel sigmoid head.  The rows of a hit come
+// from the stream-K CTAs that shared its tile.
 // Three kernels, chosen by launch_head, with the same sums in the same order
 // (so the same bits), except where noted:
 //   head_kernel       small launches with few rows: a thread per hit streams
@@ -45,7 +45,7 @@ __device__ __forceinline__ void stage_w2(float *w2, const float *__restrict__ fc
 constexpr int kManyRows = 4;  // above this many partial rows per hit, reduce them with a warp per hit
 constexpr int kSplitRows = 32;  // from this many, with four warps per hit
 
-__global__ void __launch_bounds__(kThreadsHead) head_kernel(const float *__restrict__ partials, int splits, int G,
+__global__ void __launch_bounds__(kThreadsHead) head_kernel(const float *__restrict__ partials, int G, int upt,
                                                            int n_pad, int32_t n, float s1,
                                                            const float *__restrict__ fc1_b,
                                                            const float *__restrict__ fc2_w,
@@ -71,12 +71,7 @@ __global__ void __launch_bounds__(kThreadsHead) head_kernel(const float *__restr
 
     const int64_t h = (int64_t)blockIdx.x * kThreadsHead + threadIdx.x;
     if (h >= n) return;
-    int rows = splits;
-    if (G > 0) {
-        const int64_t units = (int64_t)((n + 127) / 128) * kQuads;
-        const int64_t tile = h >> 7;
-        rows = cta_of_unit(tile * kQuads + kQuads - 1, units, G) - cta_of_unit(tile * kQuads, units, G) + 1;
-    }
+    const int rows = tile_partial_rows(h >> 7, (int64_t)((n + 127) / 128) * upt, G, upt);
 
     float h2[kN2];
 #pragma unroll
@@ -152,8 +147,8 @@ constexpr int kH1Stride = kN1 + 1;  // shared h1 rows padded: thread t reads row
 // k order (kSplit = 1: all rows in order, as head_kernel does).  More warps
 // per hit put more of the GPU on a small launch's many rows.
 template <int kHitsRows, int kSplit = 1>
-__global__ void __launch_bounds__(kThreadsRows) head_rows_kernel(const float *__restrict__ partials, int splits,
-                                                                int G, int n_pad, int32_t n, float s1,
+__global__ void __launch_bounds__(kThreadsRows) head_rows_kernel(const float *__restrict__ partials, int G,
+                                                                int upt, int n_pad, int32_t n, float s1,
                                                                 const float *__restrict__ fc1_b,
                                                                 const float *__restrict__ fc2_w,
                                                                 const float *__restrict__ fc2_b,
@@ -187,12 +182,7 @@ __global__ void __launch_bounds__(kThreadsRows) head_rows_kernel(const float *__
             if (kSplit > 1) continue;
             break;
         }
-        int rows = splits;
-        if (G > 0) {
-            const int64_t units = (int64_t)((n + 127) / 128) * kQuads;
-            const int64_t tile = h >> 7;
-            rows = cta_of_unit(tile * kQuads + kQuads - 1, units, G) - cta_of_unit(tile * kQuads, units, G) + 1;
-        }
+        const int rows = tile_partial_rows(h >> 7, (int64_t)((n + 127) / 128) * upt, G, upt);
         const int r_end = (int)((int64_t)rows * (share + 1) / kSplit);
         const float4 *p = reinterpret_cast<const float4 *>(partials + h * kN1) + lane;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -300,8 +290,8 @@ constexpr int kTileHits = 128;
 constexpr int kThreadsTile = 256;
 constexpr int kH1tStride = kTileHits + 4;  // rows of h1t: 16-byte aligned, banks shifted per k
 
-__global__ void __launch_bounds__(kThreadsTile) head_tile_kernel(const float *__restrict__ partials, int splits,
-                                                                int G, int n_pad, int32_t n, float s1,
+__global__ void __launch_bounds__(kThreadsTile) head_tile_kernel(const float *__restrict__ partials, int G,
+                                                                int upt, int n_pad, int32_t n, float s1,
                                                                 const float *__restrict__ fc1_b,
                                                                 const float *__restrict__ fc2_w,
                                                                 const float *__restrict__ fc2_b,
@@ -327,11 +317,7 @@ __global__ void __launch_bounds__(kThreadsTile) head_tile_kernel(const float *__
     }
     const int64_t h0 = (int64_t)blockIdx.x * kTileHits;
     const int64_t tile = h0 >> 7;
-    int rows = splits;
-    if (G > 0) {
-        const int64_t units = (int64_t)((n + 127) / 128) * kQuads;
-        rows = cta_of_unit(tile * kQuads + kQuads - 1, units, G) - cta_of_unit(tile * kQuads, units, G) + 1;
-    }
+    const int rows = tile_partial_rows(tile, (int64_t)((n + 127) / 128) * upt, G, upt);
     if (tile_done != nullptr) {
         // the tile's partial rows are complete once the 4 epilogue warps of each of its `rows`
         // CTAs counted theirs; the output rows were written before those CTAs read their
@@ -463,38 +449,38 @@ cudaError_t init_head_kernel_attrs() {
     return cudaFuncSetAttribute(head_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
 }
 
-bool head_counts_tiles(int32_t n, int G) {
-    return G > 0 && n > kSmallLaunch && streamk_partial_rows(n, G) <= kManyRows;
+bool head_counts_tiles(int32_t n, int G, int upt) {
+    return n > kSmallLaunch && streamk_partial_rows(n, G, upt) <= kManyRows;
 }
 
-cudaError_t launch_head(const DeviceWeights &w, const float *partials, int splits, int G, int n_pad, int32_t n,
+cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, int upt, int n_pad, int32_t n,
                         OutRows out_rows, int debug_logits, int *tile_done, int *status, int64_t timeout_ns,
                         cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     // most partial rows a hit has: many when a small launch spreads each tile over many CTAs
-    const int rows = G > 0 ? streamk_partial_rows(n, G) : splits;
+    const int rows = streamk_partial_rows(n, G, upt);
     // launched as dependents of the network kernel: the weights are staged while it finishes
     const float s1 = w.fc1_scale;
     const float *b1 = w.fc1_b, *w2 = w.fc2_w, *b2 = w.fc2_b, *wc = w.cls_w, *bc = w.cls_b, *wm = w.mic_w,
                 *bm = w.mic_b;
     if (rows > kManyRows) {
         if (rows >= kSplitRows && n <= kSmallLaunch)  // a hit's rows over 4 warps, 2 hits per block
-            return launch_pdl(head_rows_kernel<2, 4>, dim3((n + 1) / 2), dim3(kThreadsRows), 0, s, partials, splits,
-                              G, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
+            return launch_pdl(head_rows_kernel<2, 4>, dim3((n + 1) / 2), dim3(kThreadsRows), 0, s, partials, G,
+                              upt, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
         if (n <= kSmallLaunch)
-            return launch_pdl(head_rows_kernel<8>, dim3((n + 7) / 8), dim3(kThreadsRows), 0, s, partials, splits, G,
+            return launch_pdl(head_rows_kernel<8>, dim3((n + 7) / 8), dim3(kThreadsRows), 0, s, partials, G, upt,
                               n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
-        return launch_pdl(head_rows_kernel<32>, dim3((n + 31) / 32), dim3(kThreadsRows), 0, s, partials, splits, G,
+        return launch_pdl(head_rows_kernel<32>, dim3((n + 31) / 32), dim3(kThreadsRows), 0, s, partials, G, upt,
                           n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
     }
     if (n > kSmallLaunch) {
         const long long tmo = (long long)timeout_ns;
         return launch_pdl(head_tile_kernel, dim3((n + kTileHits - 1) / kTileHits), dim3(kThreadsTile), kTileSmem, s,
-                          partials, splits, G, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits,
-                          head_counts_tiles(n, G) ? tile_done : nullptr, status, tmo);
+                          partials, G, upt, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits,
+                          tile_done, status, tmo);
     }
     return launch_pdl(head_kernel, dim3((n + kThreadsHead - 1) / kThreadsHead), dim3(kThreadsHead), 0, s, partials,
-                      splits, G, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
+                      G, upt, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
 }
 
 }  // namespace emtk
