@@ -49,6 +49,9 @@ int out_stride(const emtk_ctx *c) { return c->opt.debug_logits ? 8 : 4; }
 
 int n_pad_of(int n) { return (n + 127) / 128 * 128; }
 
+// Counters of stored partial rows: four (one per 32 hits) per tile.
+size_t tile_done_words(int max_hits) { return 4 * ((size_t)(max_hits + 127) / 128 + 1); }
+
 constexpr int64_t kPartialCap = 64ll * 1024 * 1024;  // floats of the partial-sum workspace
 
 template <typename T>
@@ -379,9 +382,9 @@ cudaError_t alloc_workspace(emtk_ctx *c, bool patches) {
     }
     if (e == cudaSuccess) e = dmalloc(&c->ws.status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->ws.status, 0, sizeof(int));
-    const size_t ntiles = (size_t)(o.max_hits + 127) / 128 + 1;
-    if (e == cudaSuccess) e = dmalloc(&c->ws.tile_done, ntiles * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(c->ws.tile_done, 0, ntiles * sizeof(int));
+    const size_t ndone = tile_done_words(o.max_hits);
+    if (e == cudaSuccess) e = dmalloc(&c->ws.tile_done, ndone * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(c->ws.tile_done, 0, ndone * sizeof(int));
     return e;
 }
 
@@ -508,7 +511,6 @@ emtk_status emtk_create(const emtk_weights *w, const emtk_options *opt, int devi
             if (e == cudaSuccess) e = init_fp32_kernel_attrs();
         }
     }
-    if (e == cudaSuccess) e = init_head_kernel_attrs();
     if (e == cudaSuccess) e = alloc_workspace(c, true);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
@@ -564,7 +566,8 @@ emtk_status emtk_extract_patches(emtk_ctx *c, const float *d_adc, int32_t nwires
     if (!t) return EMTK_ERR_OOM;
     int64_t hits;
     size_t img_bytes;
-    build_table(c, &q, 0, 1, fmt, 0, *t, hits, img_bytes);
+    // with the halo, every hit in the plane has its whole window in the image
+    build_table(c, &q, 0, 1, fmt, kHalo, *t, hits, img_bytes);
     st = ensure_dimg(c, img_bytes, s);
     if (st == EMTK_OK) {
         Prof prof(c, EMTK_KERNEL_INTERVALS, s);
@@ -626,8 +629,8 @@ emtk_status emtk_check(emtk_ctx *c, emtk_stream stream) {
     if (status != 0) {
         e = cudaMemset(c->ws.status, 0, sizeof(int));
         // a launch that gave up may have left tile counters part-way
-        const size_t ntiles = (size_t)(c->opt.max_hits + 127) / 128 + 1;
-        if (e == cudaSuccess && c->ws.tile_done) e = cudaMemset(c->ws.tile_done, 0, ntiles * sizeof(int));
+        const size_t bytes = tile_done_words(c->opt.max_hits) * sizeof(int);
+        if (e == cudaSuccess && c->ws.tile_done) e = cudaMemset(c->ws.tile_done, 0, bytes);
         c->tile_mask_cap = 0;  // and tile masks: the next call reallocates and zeroes them
         if (e != cudaSuccess) return EMTK_ERR_CUDA;
         return EMTK_ERR_TIMEOUT;

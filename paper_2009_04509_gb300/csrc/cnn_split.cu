@@ -541,10 +541,10 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kBAccEmpty));
                 // this CTA's last segment of the tile: its partial row is final, count it for the head
-                if (tile_done != nullptr && (pi == np - 1 || pt == kPairsPerTile - 1)) {
+                if (tile_done != nullptr && (pi == np - 1 || pt == kPairsPerTile - 1) && tile * 128 + 32 * q4 < n) {
                     __threadfence();
                     __syncwarp();
-                    if (lane == 0) atomicAdd(tile_done + tile, 1);
+                    if (lane == 0) atomicAdd(tile_done + 4 * tile + q4, 1);
                 }
                 ++segs_done;
             }

@@ -662,10 +662,10 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kBarAccEmpty));
-                if (tile_done != nullptr) {  // this warp's rows of the tile are stored: count them for the head
+                if (tile_done != nullptr && hit0 < n) {  // this warp's rows are stored: count them for the head
                     __threadfence();
                     __syncwarp();
-                    if (lane == 0) atomicAdd(tile_done + tile, 1);
+                    if (lane == 0) atomicAdd(tile_done + 4 * tile + q4, 1);
                 }
                 ++tiles_done;
             }

@@ -124,7 +124,7 @@ struct Workspace {
     float *partials = nullptr;   // [rows][n_pad][128] of the running launch
     size_t partial_elems = 0;
     int *status = nullptr;       // device status word (bit 0: a network wait gave up, bit 1: a head wait)
-    int *tile_done = nullptr;    // [max_hits / 128 + 1] per tile: epilogue warps whose partial rows are stored
+    int *tile_done = nullptr;    // [4 tiles] per 32 hits: network CTAs whose partial rows are stored
 };
 
 struct DeviceWeights {
@@ -303,9 +303,10 @@ cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *patches, int32_
 // = streamk_partial_rows(n, G, kQuads).
 // src: 16-bit patches [n][48][48] (desc == nullptr) or the haloed interval
 // images of the hits' planes, located through desc.
-// tile_done (or null): each epilogue warp adds 1 to tile_done[tile] once its
-// partial rows of the tile are in memory (a tile is complete at 4 x its
-// partial rows).
+// tile_done (or null): epilogue warp q (hits 32 q .. 32 q + 31 of a tile) adds 1
+// to tile_done[4 tile + q] once its partial rows of the tile are in memory (32
+// hits are complete at the tile's number of partial rows); not counted for
+// quarters past n.
 // src32 (or null; 16-bit and fp8 modes, desc == nullptr): pre-cut fp32
 // patches [n][48][48] that the kernel reads itself, rounding each value as the
 // patch conversion does.
@@ -323,7 +324,7 @@ int streamk_partial_rows(int32_t n, int G, int upt);
 // Sum of partials + bias + ReLU, dense-2, heads; hit h's scores where out_rows says.  Partial
 // rows: the stream-K contributors of the hit's tile (G CTAs, upt units per
 // tile).  With tile_done (launches for which head_counts_tiles(n, G, upt)
-// holds), a tile's head starts once the tile's counter is complete instead of
+// holds), the head of 32 hits starts once their counter is complete instead of
 // after the whole network kernel, gives up when bit 0 of *status is set or
 // after timeout_ns (setting bit 1), and sets the counter back to zero.
 bool head_counts_tiles(int32_t n, int G, int upt);
@@ -333,7 +334,6 @@ cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, in
 
 // Kernel attributes (dynamic shared memory), set once per device at create.
 cudaError_t init_fp32_kernel_attrs();
-cudaError_t init_head_kernel_attrs();
 cudaError_t init_tc_kernel_attrs();
 
 // Host helpers for the tensor-core weights (cnn_tc.cu, cnn_split.cu).
