@@ -164,10 +164,21 @@ constexpr float kSplitPatchScale = 0.0625f;  // s_p: 2^-4
 // CTA of that one has started and executed pdl_trigger, or finished), so its
 // set-up overlaps that kernel's tail; before it reads anything that kernel
 // (or an earlier one) wrote, it executes pdl_wait, which returns once the
-// previous kernel has completed and its writes are visible.
+// previous kernel has completed and its writes are visible.  Every kernel of the
+// chain executes pdl_wait before it completes (in one block at least), so the
+// completion of one implies that of all before it.  A kernel that lets its
+// successor read caller buffers before pdl_wait starts with pdl_begin: the
+// successor is then scheduled only once what wrote those buffers has completed.
+// The first kernel of a call is launched this way too: back-to-back calls overlap
+// its scheduling with the head of the call before (256 hits of one plane, bf16:
+// 28.8 -> 25.9 us per call).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_begin() {
+    pdl_wait();
+    pdl_trigger();
+}
 #endif
 
 template <typename... KArgs, typename... Args>

@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(kThreadsRows) head_rows_kernel(const float *__
     __shared__ __align__(16) float w2[kN1][kN2];
     __shared__ __align__(16) float wc[kN2][kNC + 1];
     __shared__ float b2[kN2];
+    pdl_trigger();  // the next call's first kernel may be scheduled; it waits for this one
     stage_w2<kThreadsRows>(&w2[0][0], fc2_w);
     for (int i = threadIdx.x; i < kN2 * kNC; i += blockDim.x) wc[i / kNC][i % kNC] = cls_w[i];
     for (int i = threadIdx.x; i < kN2; i += blockDim.x) {
@@ -213,6 +214,7 @@ __global__ void __launch_bounds__(kThreadsHits) head_hits_kernel(const float *__
     __shared__ float wc[kN2][kNC + 1];
     __shared__ int go;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_trigger();  // the next call's first kernel may be scheduled; it waits for this one
     stage_w2<kThreadsHits>(&w2[0][0], fc2_w);
     for (int i = tid; i < kN2 * kNC; i += kThreadsHits) wc[i / kNC][i % kNC] = cls_w[i];
     for (int i = tid; i < kN2; i += kThreadsHits) wc[i][kNC] = mic_w[i];
@@ -242,6 +244,9 @@ __global__ void __launch_bounds__(kThreadsHits) head_hits_kernel(const float *__
                 __nanosleep(200);
             }
             tile_done[blockIdx.x] = 0;  // every row is counted (or the launch gave up): zero for the next launch
+            // one block lasts as long as the network kernel, so that the completion of this
+            // kernel implies that one's
+            if (blockIdx.x == gridDim.x - 1) pdl_wait();
             go = ok;
         }
         __syncthreads();
