@@ -763,8 +763,7 @@ emtk_status emtk_find_hits(emtk_ctx *c, emtk_hitfind_request *reqs, int32_t nreq
     if (!c || nreq < 0 || (nreq > 0 && !reqs)) return EMTK_ERR_ARG;
     // the most runs a plane can hold: one per two ticks on every wire
     auto max_runs = [](const emtk_hitfind_request &q) { return (int64_t)q.nwires * ((q.nticks + 1) / 2); };
-    // scratch (the partial-sum workspace): plane totals in its first 256 bytes, then the
-    // group's per-wire scratch
+    // scratch: the partial-sum workspace past its first 256 bytes
     const size_t scratch_bytes = c->ws.partial_elems * sizeof(float) - 256;
     const int64_t unit_cap = find_hits_unit_cap(scratch_bytes);
     // a plane's units: wire segments of kSegTicks ticks (none without ticks)
@@ -791,7 +790,6 @@ emtk_status emtk_find_hits(emtk_ctx *c, emtk_hitfind_request *reqs, int32_t nreq
         if (host_alloc(&h, sizeof(int32_t) * kMaxHfPlanes) != cudaSuccess) return EMTK_ERR_OOM;
         c->h_totals = static_cast<int32_t *>(h);
     }
-    int32_t *totals = reinterpret_cast<int32_t *>(c->ws.partials);
     void *scratch = reinterpret_cast<char *>(c->ws.partials) + 256;
     int32_t i = 0;
     while (i < nreq) {
@@ -835,10 +833,11 @@ emtk_status emtk_find_hits(emtk_ctx *c, emtk_hitfind_request *reqs, int32_t nreq
         int32_t *next = c->hf_sums + (int64_t)(1 - c->hf_parity) * c->hf_sums_cap;
         {
             Prof prof(c, EMTK_KERNEL_HITFIND, s, U > 0 ? 2 : 0);  // find, then place
-            e = launch_find_hits(t, U, scratch, cur, next, c->hf_sums_cap, totals, s);
+            // the kernels write the planes' counts straight to pinned memory
+            std::memset(c->h_totals, 0, sizeof(int32_t) * kMaxHfPlanes);
+            e = launch_find_hits(t, U, scratch, cur, next, c->hf_sums_cap, c->h_totals, s);
         }
         if (e == cudaSuccess && U > 0) c->hf_parity ^= 1;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(c->h_totals, totals, sizeof(int32_t) * t.n, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) {
             // the launch or the kernels may have stopped before the place kernel cleared

@@ -227,7 +227,7 @@ struct emtk_ctx {
     } stage[2];
     cudaStream_t copy_stream = nullptr;
     uint64_t host_calls = 0;
-    int32_t *h_totals = nullptr;  // pinned: emtk_find_hits' per-plane counts (kMaxHfPlanes)
+    int32_t *h_totals = nullptr;  // pinned, written by the kernels: emtk_find_hits' per-plane counts (kMaxHfPlanes)
     // emtk_find_hits' chunk sums: two halves of hf_sums_cap, used in turn; each
     // launch clears the other half for the next one
     int32_t *hf_sums = nullptr;
@@ -300,7 +300,8 @@ cudaError_t launch_hit_desc(const ReqTable &t, int64_t g0, int32_t count, HitDes
 // holds per-unit run counts and run slots; find_hits_unit_cap gives the most
 // units that scratch_bytes holds.  The chunk sums live in sums_cur (zero on
 // entry, find_hits_chunks(t, U) of them); the launch zeroes sums_next[0, cap)
-// for the next launch.  totals[r] receives plane r's hit count.
+// for the next launch.  totals[r] (device-accessible, e.g. pinned host memory)
+// receives plane r's hit count; it is not written when nunits is 0.
 int64_t find_hits_unit_cap(size_t scratch_bytes);
 int64_t find_hits_chunks(const HfTable &t, int64_t nunits);
 cudaError_t launch_find_hits(const HfTable &t, int64_t nunits, void *scratch, int32_t *sums_cur, int32_t *sums_next,

@@ -21,15 +21,21 @@
 //                    scratch slots, writes its run count and adds it to its
 //                    chunk's sum (chunks: kHfChunk consecutive units of one
 //                    plane);
-//   hf_place_kernel  one CTA per chunk, a thread per unit: a unit's offset in
-//                    its plane is the sum of the plane's earlier chunks plus
-//                    a block scan of the chunk's counts.  The chunk's runs in
-//                    the slots are then shared out evenly: thread i copies
-//                    runs i, i + kHfChunk, ... of the chunk (its unit found by
-//                    binary search of the scanned counts), so consecutive
-//                    threads write consecutive hits.  A unit with more runs
-//                    than slots is scanned again by a warp and written
-//                    directly.  The plane's last unit writes its total.
+//   hf_place_kernel  one CTA per chunk: a unit's offset in its plane is the sum
+//                    of the plane's earlier chunks (one warp) plus a scan of
+//                    the chunk's counts (another, a lane per unit).  The
+//                    chunk's runs in the slots are then shared out evenly:
+//                    thread i copies runs i, i + kPlaceThreads, ... of the
+//                    chunk (its unit found by binary search of the scanned
+//                    counts), so consecutive threads write consecutive hits.
+//                    A unit with more runs than slots is scanned again by a
+//                    warp and written directly.  The plane's last unit writes
+//                    its total, straight into the caller's pinned host memory
+//                    (a copy after the kernel cost 6 us of the call).  Bound
+//                    by its chain of round trips to L2, so a chunk is small
+//                    enough for one run per thread: with 128 units per CTA
+//                    (360 CTAs, 4 rounds on the full event) it ended 9 us after
+//                    the find kernel, with 32 units 5 us after it.
 // The chunk sums start at zero: the place kernel of the launch before cleared
 // them (they alternate between two arrays of the context).  The plane is read
 // once from HBM (plus units with more than kRunSlots runs).  No kernel waits
@@ -47,7 +53,8 @@ namespace {
 constexpr int kHfWarps = 4;     // warps (units) per CTA of the find kernel
 constexpr int kHfSub = 4;       // 128-tick blocks loaded per step (4 loads in flight per lane)
 constexpr int kRunSlots = 128;  // runs per unit kept in scratch (more: the unit is scanned again)
-constexpr int kHfChunk = 128;   // units per chunk: threads per CTA of the place kernel
+constexpr int kHfChunk = 32;    // units per chunk (one CTA of the place kernel): a lane each
+constexpr int kPlaceThreads = 128;
 constexpr unsigned kFull = 0xffffffffu;
 static_assert(kSegTicks % (128 * kHfSub) == 0, "a segment is whole load blocks");
 
@@ -267,18 +274,18 @@ __global__ void __launch_bounds__(kHfWarps * 32) hf_find_kernel(const __grid_con
 }
 
 // One CTA per chunk (blockIdx.x = the chunk's index in the group).
-__global__ void __launch_bounds__(kHfChunk) hf_place_kernel(const __grid_constant__ HfTable t, int64_t nunits,
-                                                             const int32_t *__restrict__ chunk_sum,
-                                                             const int32_t *__restrict__ counts,
-                                                             const Run *__restrict__ slots,
-                                                             int32_t *__restrict__ total,
-                                                             int32_t *__restrict__ sums_next, int64_t cap) {
-    constexpr int kWarps = kHfChunk / 32;
+__global__ void __launch_bounds__(kPlaceThreads) hf_place_kernel(const __grid_constant__ HfTable t, int64_t nunits,
+                                                                  const int32_t *__restrict__ chunk_sum,
+                                                                  const int32_t *__restrict__ counts,
+                                                                  const Run *__restrict__ slots,
+                                                                  int32_t *__restrict__ total,
+                                                                  int32_t *__restrict__ sums_next, int64_t cap) {
+    constexpr int kWarps = kPlaceThreads / 32;
+    static_assert(kHfChunk == 32 && kWarps >= 2, "one warp scans the chunk, another sums the chunks before it");
     __shared__ int32_t cum[kHfChunk + 1];  // runs copied from the slots before each unit
-    __shared__ int32_t out[kHfChunk];      // each unit's offset in its plane
-    __shared__ uint64_t warp_tot[kWarps];
-    __shared__ int32_t base_sh, nover_sh;
-    __shared__ int32_t over[kHfChunk];     // units with more runs than slots
+    __shared__ int32_t out[kHfChunk];      // each unit's offset in its chunk
+    __shared__ int32_t base_sh;            // the chunk's offset in its plane
+    __shared__ uint32_t over_sh;           // units with more runs than slots
     __shared__ float4 stash[kWarps][32 * kHfSub];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (blockIdx.x == 0 && tid < t.n) {  // planes without units
@@ -287,7 +294,7 @@ __global__ void __launch_bounds__(kHfChunk) hf_place_kernel(const __grid_constan
     }
     // the next launch's chunk sums start at zero (this call's find kernel uses the
     // other array, and the last reader of this one finished before it started)
-    for (int64_t i = (int64_t)blockIdx.x * kHfChunk + tid; i < cap; i += (int64_t)gridDim.x * kHfChunk)
+    for (int64_t i = (int64_t)blockIdx.x * kPlaceThreads + tid; i < cap; i += (int64_t)gridDim.x * kPlaceThreads)
         sums_next[i] = 0;
     int r = 0;  // the chunk's plane: the last with chunk0 <= blockIdx.x
     while (r + 1 < t.n && t.r[r + 1].chunk0 <= (int64_t)blockIdx.x) ++r;
@@ -296,38 +303,37 @@ __global__ void __launch_bounds__(kHfChunk) hf_place_kernel(const __grid_constan
     const int64_t pend = r + 1 < t.n ? t.r[r + 1].unit0 : nunits;
     const int64_t c = (int64_t)blockIdx.x - d.chunk0;
     const int64_t first = d.unit0 + c * kHfChunk;
-    const int64_t u = first + tid;
-    const int32_t n = u < pend ? counts[u] : 0;
-    const int32_t m = n <= kRunSlots ? n : 0;  // runs copied from the slots
-    if (tid == 0) nover_sh = 0;
-    if (warp == 0) {  // the plane's chunks before this one
+    int32_t n = 0, incl_n = 0;
+    if (warp == 0) {
+        n = first + lane < pend ? counts[first + lane] : 0;
+        const int32_t m = n <= kRunSlots ? n : 0;  // runs copied from the slots
+        incl_n = n;
+        int32_t incl_m = m;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t yn = __shfl_up_sync(kFull, incl_n, o), ym = __shfl_up_sync(kFull, incl_m, o);
+            if (lane >= o) {
+                incl_n += yn;
+                incl_m += ym;
+            }
+        }
+        out[lane] = incl_n - n;
+        cum[lane] = incl_m - m;
+        if (lane == 31) cum[kHfChunk] = incl_m;
+        const uint32_t over = __ballot_sync(kFull, n > kRunSlots);
+        if (lane == 0) over_sh = over;
+    } else if (warp == 1) {  // the plane's chunks before this one
         int32_t acc = 0;
         for (int64_t k = lane; k < c; k += 32) acc += chunk_sum[d.chunk0 + k];
         acc = (int32_t)__reduce_add_sync(kFull, (uint32_t)acc);
         if (lane == 0) base_sh = acc;
     }
-    // block scan of (n, m) packed in 64 bits: both sums stay below 2^31
-    uint64_t incl = ((uint64_t)(uint32_t)n << 32) | (uint32_t)m;
-    const uint64_t own = incl;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_tot[warp] = incl;
     __syncthreads();
-    uint64_t excl = incl - own;
-    for (int w = 0; w < warp; ++w) excl += warp_tot[w];
-    const int32_t off = base_sh + (int32_t)(excl >> 32);
-    out[tid] = off;
-    cum[tid] = (int32_t)(uint32_t)excl;
-    if (tid == kHfChunk - 1) cum[kHfChunk] = (int32_t)(uint32_t)(excl + own);
-    if (n > kRunSlots) over[atomicAdd(&nover_sh, 1)] = tid;
-    if (u == pend - 1) total[r] = off + n;
-    __syncthreads();
+    const int32_t base = base_sh;
+    if (warp == 0 && first + lane == pend - 1) total[r] = base + incl_n;
     // the slots' runs, shared out evenly
     const int32_t nrun = cum[kHfChunk];
-    for (int32_t i = tid; i < nrun; i += kHfChunk) {
+    for (int32_t i = tid; i < nrun; i += kPlaceThreads) {
         int lo = 0, hi = kHfChunk - 1;  // the unit j with cum[j] <= i < cum[j + 1]
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -338,13 +344,15 @@ __global__ void __launch_bounds__(kHfChunk) hf_place_kernel(const __grid_constan
         }
         const int32_t k = i - cum[lo];
         const int64_t uj = first + lo;
-        put_hit(d, unit_of(d, uj).wire, out[lo] + k, slots[uj * kRunSlots + k]);
+        put_hit(d, unit_of(d, uj).wire, base + out[lo] + k, slots[uj * kRunSlots + k]);
     }
     // units with more runs than slots: a warp each, scanned again
-    for (int q = warp; q < nover_sh; q += kWarps) {
-        const int j = over[q];
+    int q = 0;
+    for (uint32_t over = over_sh; over; over &= over - 1, ++q) {
+        if (q % kWarps != warp) continue;
+        const int j = __ffs(over) - 1;
         const Unit unit = unit_of(d, first + j);
-        const int32_t oj = out[j];
+        const int32_t oj = base + out[j];
         const Src src{unit.row, unit.t1, reinterpret_cast<float *>(stash[warp]), 0, 0};
         scan_unit(unit, src, d.nticks, d.thr, lane, [&](int32_t k, const Run &run) { put_hit(d, unit.wire, oj + k, run); });
     }
@@ -367,7 +375,7 @@ int64_t find_hits_chunks(const HfTable &t, int64_t nunits) {
 
 cudaError_t launch_find_hits(const HfTable &t_in, int64_t nunits, void *scratch, int32_t *sums_cur, int32_t *sums_next,
                              int64_t cap, int32_t *totals, cudaStream_t s) {
-    if (nunits <= 0) return cudaMemsetAsync(totals, 0, sizeof(int32_t) * kMaxHfPlanes, s);
+    if (nunits <= 0) return cudaSuccess;
     HfTable t = t_in;
     int64_t nchunks = 0;
     for (int r = 0; r < t.n; ++r) {
@@ -384,7 +392,7 @@ cudaError_t launch_find_hits(const HfTable &t_in, int64_t nunits, void *scratch,
     if (e != cudaSuccess) return e;
     const int32_t *cc = counts;
     const Run *cs = slots;
-    return launch_pdl(hf_place_kernel, dim3((unsigned)nchunks), dim3(kHfChunk), 0, s, t, nunits,
+    return launch_pdl(hf_place_kernel, dim3((unsigned)nchunks), dim3(kPlaceThreads), 0, s, t, nunits,
                       static_cast<const int32_t *>(sums_cur), cc, cs, totals, sums_next, cap);
 }
 
