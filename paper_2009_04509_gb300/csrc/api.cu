@@ -201,11 +201,14 @@ emtk_status run_network(emtk_ctx *c, const void *patches, const HitDesc *desc, i
     const bool tc = tensor_precision(c->opt.precision);
     const int upt = tc ? kQuads : kPos / 2;
     // one persistent CTA per SM (stream-K), fewer if the partial rows would not fit
-    int G = c->sm_count;
-    while (G > 1 && streamk_partial_rows(n, G, upt) > max_rows) G /= 2;
+    int G = c->sm_count, rows = streamk_partial_rows(n, G, upt);
+    while (G > 1 && rows > max_rows) {
+        G /= 2;
+        rows = streamk_partial_rows(n, G, upt);
+    }
     // the head of a large launch takes each tile as soon as its partial rows are stored
     // (the tensor-core kernels count them; no kernel of the fp32 path waits on another)
-    int *tile_done = tc && head_counts_tiles(n, G, upt) ? c->ws.tile_done : nullptr;
+    int *tile_done = tc && head_counts_tiles(n, rows) ? c->ws.tile_done : nullptr;
     {
         Prof prof(c, EMTK_KERNEL_NETWORK, s);
         e = tc ? launch_cnn_tc(c->w, patches, desc, tc_mode(c->opt.precision), n, G, c->ws.partials, n_pad,
@@ -215,7 +218,7 @@ emtk_status run_network(emtk_ctx *c, const void *patches, const HitDesc *desc, i
     if (e != cudaSuccess) return cuda_status(e);
     {
         Prof prof(c, EMTK_KERNEL_HEAD, s);
-        e = launch_head(c->w, c->ws.partials, G, upt, n_pad, n, out_rows, c->opt.debug_logits, tile_done,
+        e = launch_head(c->w, c->ws.partials, G, upt, rows, n_pad, n, out_rows, c->opt.debug_logits, tile_done,
                         c->ws.status, c->opt.wait_timeout_ns, s);
     }
     count_launch(c, n);

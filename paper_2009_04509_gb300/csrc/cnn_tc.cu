@@ -805,14 +805,19 @@ cudaError_t prepare_tc_weights(DeviceWeights &w, const emtk_weights &hw, TcMode 
 }
 
 // Partial-sum rows a stream-K launch over G CTAs needs: the largest number
-// of CTAs that share one tile.
+// of CTAs that share one tile, i.e. one more than the most CTA boundaries that
+// lie strictly inside a tile.  A pass over the G - 1 boundaries (in order, so a
+// tile's are consecutive), not over the tiles.
 int streamk_partial_rows(int32_t n, int G, int upt) {
-    const int m_tiles = (n + 127) / 128;
-    const int64_t units = (int64_t)m_tiles * upt;
-    int rows = 1;
-    for (int t = 0; t < m_tiles; ++t) {
-        const int r = tile_partial_rows(t, units, G, upt);
-        rows = r > rows ? r : rows;
+    const int64_t units = (int64_t)((n + 127) / 128) * upt;
+    int rows = 1, in_tile = 1;
+    int64_t tile = -1;
+    for (int c = 1; c < G; ++c) {
+        const int64_t u = unit_begin(c, units, G);
+        if (u % upt == 0) continue;  // between tiles
+        in_tile = u / upt == tile ? in_tile + 1 : 2;
+        tile = u / upt;
+        rows = in_tile > rows ? in_tile : rows;
     }
     return rows;
 }

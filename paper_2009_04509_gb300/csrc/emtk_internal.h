@@ -339,8 +339,8 @@ int streamk_partial_rows(int32_t n, int G, int upt);
 // holds), the head of 32 hits starts once their counter is complete instead of
 // after the whole network kernel, gives up when bit 0 of *status is set or
 // after timeout_ns (setting bit 1), and sets the counter back to zero.
-bool head_counts_tiles(int32_t n, int G, int upt);
-cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, int upt, int n_pad,
+bool head_counts_tiles(int32_t n, int rows);
+cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, int upt, int rows, int n_pad,
                         int32_t n, OutRows out_rows, int debug_logits, int *tile_done, int *status,
                         int64_t timeout_ns, cudaStream_t s);
 

@@ -344,16 +344,14 @@ __global__ void __launch_bounds__(kThreadsHits) head_hits_kernel(const float *__
 
 }  // namespace
 
-bool head_counts_tiles(int32_t n, int G, int upt) {
-    return n > kSmallLaunch && streamk_partial_rows(n, G, upt) <= kManyRows;
+bool head_counts_tiles(int32_t n, int rows) {
+    return n > kSmallLaunch && rows <= kManyRows;
 }
 
-cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, int upt, int n_pad, int32_t n,
+cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, int upt, int rows, int n_pad, int32_t n,
                         OutRows out_rows, int debug_logits, int *tile_done, int *status, int64_t timeout_ns,
                         cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    // most partial rows a hit has: many when a small launch spreads each tile over many CTAs
-    const int rows = streamk_partial_rows(n, G, upt);
     // launched as dependents of the network kernel: the weights are staged while it finishes
     const float s1 = w.fc1_scale;
     const float *b1 = w.fc1_b, *w2 = w.fc2_w, *b2 = w.fc2_b, *wc = w.cls_w, *bc = w.cls_b, *wm = w.mic_w,

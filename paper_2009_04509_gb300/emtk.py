@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -59,6 +60,13 @@ class emtk_hitfind_request(ctypes.Structure):
     _fields_ = [("d_adc", _vp), ("nwires", ctypes.c_int32), ("nticks", ctypes.c_int32), ("ld", ctypes.c_int64),
                 ("threshold", ctypes.c_float), ("capacity", ctypes.c_int32), ("d_hits", _vp), ("d_info", _vp),
                 ("n_found", ctypes.c_int32), ("reserved", ctypes.c_int32)]
+
+
+# The request structures as struct formats (native alignment): filling a whole structure
+# at once takes a third of the time of its fields one by one.
+_REQUEST = struct.Struct("@PiiqPiP")
+_HITFIND = struct.Struct("@PiiqfiPPii")
+assert _REQUEST.size == ctypes.sizeof(emtk_request) and _HITFIND.size == ctypes.sizeof(emtk_hitfind_request)
 
 
 class EmtkError(RuntimeError):
@@ -143,13 +151,12 @@ def _check(rc: int, what: str) -> int:
 
 def _ptr(t) -> int:
     """Device pointer of a torch tensor (or a raw int)."""
-    if t is None:
-        return 0
-    if isinstance(t, int):
-        return t
-    if not t.is_contiguous():
-        raise ValueError("tensor must be contiguous")
-    return t.data_ptr()
+    try:
+        if t.is_contiguous():
+            return t.data_ptr()
+    except AttributeError:
+        return 0 if t is None else int(t)
+    raise ValueError("tensor must be contiguous")
 
 
 def _stream(stream) -> int:
@@ -205,9 +212,15 @@ def make_requests(items) -> ctypes.Array:
     """items: iterable of (adc, nticks, hits, scores) tensors."""
     items = list(items)
     arr = (emtk_request * max(1, len(items)))()
+    at = 0
     for i, (adc, nticks, hits, scores) in enumerate(items):
-        arr[i] = emtk_request(_ptr(adc), int(adc.shape[0]), int(nticks), int(adc.shape[1]), _ptr(hits),
-                              int(hits.shape[0]), _ptr(scores))
+        nwires, ld = adc.shape
+        try:
+            _REQUEST.pack_into(arr, at, _ptr(adc), nwires, int(nticks), ld, _ptr(hits), hits.shape[0], _ptr(scores))
+        except struct.error:  # a number that ctypes would wrap
+            arr[i] = emtk_request(_ptr(adc), int(nwires), int(nticks), int(ld), _ptr(hits), int(hits.shape[0]),
+                                  _ptr(scores))
+        at += _REQUEST.size
     return arr
 
 
@@ -267,18 +280,22 @@ def emtk_find_hits(ctx, planes, stream=None) -> list:
     or None).  info columns: start, end, then peak and charge as float32 bits
     (``info[:, 2:].view(torch.float32)``).  Returns the number of hits found per
     plane (which may exceed a plane's capacity); the call synchronises the stream."""
-    reqs = (emtk_hitfind_request * max(1, len(planes)))()
+    n = len(planes)
+    reqs = (emtk_hitfind_request * max(1, n))()
+    at = 0
     for i, (adc, nticks, thr, hits, info) in enumerate(planes):
-        q = reqs[i]
-        q.d_adc = _ptr(adc)
-        q.nwires, q.ld = adc.shape
-        q.nticks = int(nticks)
-        q.threshold = float(thr)
-        q.capacity = hits.shape[0]
-        q.d_hits = _ptr(hits)
-        q.d_info = _ptr(info) if info is not None else None
-    _check(load_library().emtk_find_hits(ctx, reqs, len(planes), _stream(stream)), "emtk_find_hits")
-    return [int(reqs[i].n_found) for i in range(len(planes))]
+        nwires, ld = adc.shape
+        try:
+            _HITFIND.pack_into(reqs, at, _ptr(adc), nwires, int(nticks), ld, thr, hits.shape[0], _ptr(hits),
+                               _ptr(info), 0, 0)
+        except (struct.error, OverflowError):  # a number that ctypes would wrap, or round to infinity
+            q = reqs[i]
+            q.d_adc, q.nwires, q.nticks, q.ld = _ptr(adc), int(nwires), int(nticks), int(ld)
+            q.threshold, q.capacity = float(thr), int(hits.shape[0])
+            q.d_hits, q.d_info = _ptr(hits), _ptr(info)
+        at += _HITFIND.size
+    _check(load_library().emtk_find_hits(ctx, reqs, n, _stream(stream)), "emtk_find_hits")
+    return [q[8] for q in _HITFIND.iter_unpack(reqs)][:n]
 
 
 def emtk_get_fp8_scales(ctx) -> tuple:
