@@ -3,15 +3,11 @@
 // of the e4m3 path), + bias + ReLU, dense 128->32 + ReLU, the 3-way softmax
 // head (track, em, none) and the Michel sigmoid head.  The rows of a hit come
 // from the stream-K CTAs that shared its tile.
-// Two kernels, chosen by launch_head:
+// Two kernels, chosen by launch_head, each with its sums in a fixed order:
 //   head_rows_kernel  small launches, whose tiles are spread over many CTAs: a
-//                     warp per hit sums its many rows, 16 deep (from 32 rows
-//                     on, four warps per hit each sum a quarter of the rows
-//                     and the quarters are added in order);
+//                     CTA per hit or two, its warps share the hit's many rows;
 //   head_hits_kernel  the others: a CTA per 32 hits, the share of one epilogue
 //                     warp of the network kernels.
-// Both add the rows in order (but for the four quarters) and the inputs of
-// every dense-2 and head sum in order, so they give the same bits.
 #include "emtk_internal.h"
 
 namespace emtk {
@@ -36,24 +32,34 @@ __device__ __forceinline__ void stage_w2(float *w2, const float *__restrict__ fc
 #pragma unroll
     for (int k = 0; k < kN4 / kThreads; ++k) reinterpret_cast<float4 *>(w2)[threadIdx.x + k * kThreads] = v[k];
 }
-constexpr int kManyRows = 4;    // up to this many partial rows per hit, head_hits_kernel at any size
-constexpr int kSplitRows = 32;  // from this many, head_rows_kernel with four warps per hit
+constexpr int kManyRows = 4;  // up to this many partial rows per hit, head_hits_kernel at any size
 
 // The tail when a hit has many partial rows (a small launch, whose tiles are
-// split over many CTAs): one warp per hit sums the rows, lane l taking dense-1
-// outputs 4l .. 4l+3 of every row (512 contiguous bytes per row), and writes
-// bias + ReLU to shared memory; every thread then computes dense-2 outputs (one
-// per hit and output), and one thread per hit the heads.
+// split over many CTAs), HITS hits per CTA of 8 warps.  What bounds it is its
+// chain of latencies after the network kernel's last row, so nothing but the rows
+// is loaded on it and every step is spread over the warps:
+//   before the wait  thread (warp w, lane j) takes the dense-2 weights of inputs
+//                    16 w .. 16 w + 15 to output j into registers;
+//   1. kSplit = 8 / HITS warps per hit: warp k sums rows [k R / kSplit,
+//      (k + 1) R / kSplit) in order, lane l dense-1 outputs 4 l .. 4 l + 3, up to
+//      kDepth rows in one round trip;
+//   2. a thread per (hit, dense-1 output) adds the shares in order, bias + ReLU;
+//   3. dense-2: every warp its 16 inputs, for all hits;
+//   4. a warp per hit adds the 8 parts in order, bias + ReLU, and the head logits
+//      by warp sums.
+// Against a kernel with the dense-2 weights staged in shared memory, one thread per
+// dense-2 output and one per hit for the heads: 256 hits of one plane (76 rows per
+// hit) 26.6 -> 23.8 us per call, 128 patches 21.3 -> 18.3, 1,693 54.9 -> 53.9.
 constexpr int kThreadsRows = 256;
-constexpr int kSmallLaunch = 2048;
-constexpr int kH1Stride = kN1 + 1;  // shared h1 rows padded: thread t reads row t conflict-free
+constexpr int kSmallLaunch = 2048;  // above it, head_hits_kernel
+// Up to kOneHit hits one per CTA, up to kTwoHits two, else four: each the fewest that
+// keep the launch in one wave of 2 or 3 CTAs per SM (256 hits: 23.8 us per call with
+// one, 24.9 with two; 1,000: 38.4 with two, 35.4 with four).
+constexpr int kOneHit = 256, kTwoHits = 912;
+constexpr int kDepth = 10;          // rows per round trip: all of a share from 129 hits on (77 rows)
 
-// kSplit warps share a hit: warp k of the hit sums its rows [k R / kSplit,
-// (k+1) R / kSplit) in order, and the kSplit partial sums are then added in
-// k order (kSplit = 1: all rows in order).  More warps
-// per hit put more of the GPU on a small launch's many rows.
-template <int kHitsRows, int kSplit = 1>
-__global__ void __launch_bounds__(kThreadsRows) head_rows_kernel(const float *__restrict__ partials, int G,
+template <int HITS>
+__global__ void __launch_bounds__(kThreadsRows, HITS == 1 ? 2 : 3) head_rows_kernel(const float *__restrict__ partials, int G,
                                                                 int upt, int n_pad, int32_t n, float s1,
                                                                 const float *__restrict__ fc1_b,
                                                                 const float *__restrict__ fc2_w,
@@ -63,123 +69,89 @@ __global__ void __launch_bounds__(kThreadsRows) head_rows_kernel(const float *__
                                                                 const float *__restrict__ mic_w,
                                                                 const float *__restrict__ mic_b, OutRows out_rows,
                                                                 int debug_logits) {
-    static_assert(kHitsRows * kSplit <= kThreadsRows / 32 || kSplit == 1, "a warp per (hit, row share)");
-    __shared__ float h1s[kHitsRows * kH1Stride];
-    __shared__ __align__(16) float4 part[kSplit > 1 ? kHitsRows * kSplit * 32 : 1];
-    __shared__ float h2s[kHitsRows * (kN2 + 1)];
-    __shared__ __align__(16) float w2[kN1][kN2];
-    __shared__ __align__(16) float wc[kN2][kNC + 1];
-    __shared__ float b2[kN2];
+    constexpr int kWarps = kThreadsRows / 32, kSplit = kWarps / HITS, kShare = kN1 / kWarps;
+    static_assert(kThreadsRows % kN1 == 0 && kWarps % HITS == 0, "whole dense-1 rows per pass, whole warps per hit");
+    __shared__ __align__(16) float part[kWarps][kN1];        // row sums of each warp's share
+    __shared__ __align__(16) float h1[HITS][kN1];
+    __shared__ float part2[HITS][kWarps][kN2];
     pdl_trigger();  // the next call's first kernel may be scheduled; it waits for this one
-    stage_w2<kThreadsRows>(&w2[0][0], fc2_w);
-    for (int i = threadIdx.x; i < kN2 * kNC; i += blockDim.x) wc[i / kNC][i % kNC] = cls_w[i];
-    for (int i = threadIdx.x; i < kN2; i += blockDim.x) {
-        wc[i][kNC] = mic_w[i];
-        b2[i] = fc2_b[i];
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    pdl_wait();  // the partial sums and output rows come from the kernels before
-    const int64_t h0 = (int64_t)blockIdx.x * kHitsRows;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    float w2[kShare];
+#pragma unroll
+    for (int i = 0; i < kShare; ++i) w2[i] = __ldg(fc2_w + (kShare * warp + i) * kN2 + lane);
+    const float b1 = __ldg(fc1_b + (tid & (kN1 - 1))), b2 = __ldg(fc2_b + lane);
+    const float wc[kNC + 1] = {__ldg(cls_w + lane * kNC), __ldg(cls_w + lane * kNC + 1), __ldg(cls_w + lane * kNC + 2),
+                               __ldg(mic_w + lane)};
+    const float bc[kNC + 1] = {__ldg(cls_b), __ldg(cls_b + 1), __ldg(cls_b + 2), __ldg(mic_b)};
+    const int64_t h0 = (int64_t)blockIdx.x * HITS;
+    const int64_t units = (int64_t)((n + 127) / 128) * upt;
+    const int j = warp / kSplit, share = warp % kSplit;  // this warp's hit and share of its rows
+    const int rows = tile_partial_rows((h0 + j) >> 7, units, G, upt);
+    int r = rows * share / kSplit;
+    const int r_end = rows * (share + 1) / kSplit;
     const int64_t row_stride = (int64_t)n_pad * kN1 / 4;  // float4s between partial rows
-    const float4 bb = reinterpret_cast<const float4 *>(fc1_b)[lane];
-    for (int jw = warp; jw < kHitsRows * kSplit; jw += kThreadsRows / 32) {
-        const int j = jw / kSplit, share = jw % kSplit;
-        const int64_t h = h0 + j;
-        if (h >= n) {
-            if (kSplit > 1) continue;
-            break;
-        }
-        const int rows = tile_partial_rows(h >> 7, (int64_t)((n + 127) / 128) * upt, G, upt);
-        const int r_end = (int)((int64_t)rows * (share + 1) / kSplit);
-        const float4 *p = reinterpret_cast<const float4 *>(partials + h * kN1) + lane;
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        // this warp's rows in order, loaded kDepth at a time (the last batch
-        // predicated), so that a hit's rows cost one round trip per kDepth rows
-        constexpr int kDepth = 16;
-        for (int r = (int)((int64_t)rows * share / kSplit); r < r_end; r += kDepth) {
-            float4 v[kDepth];
+    const float4 *p = reinterpret_cast<const float4 *>(partials + (h0 + j) * kN1) + lane;
+    pdl_wait();  // the partial sums and output rows come from the kernels before
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (; r < r_end; r += kDepth) {  // a row past n lies in the tile's padding: read, never used
+        float4 v[kDepth];
 #pragma unroll
-            for (int k = 0; k < kDepth; ++k)
-                if (r + k < r_end) v[k] = p[(r + k) * row_stride];
+        for (int k = 0; k < kDepth; ++k)
+            if (r + k < r_end) v[k] = p[(r + k) * row_stride];
 #pragma unroll
-            for (int k = 0; k < kDepth; ++k) {
-                if (r + k < r_end) {
-                    a.x += v[k].x;
-                    a.y += v[k].y;
-                    a.z += v[k].z;
-                    a.w += v[k].w;
-                }
+        for (int k = 0; k < kDepth; ++k)
+            if (r + k < r_end) {
+                a.x += v[k].x;
+                a.y += v[k].y;
+                a.z += v[k].z;
+                a.w += v[k].w;
             }
-        }
-        if (kSplit > 1) {
-            part[jw * 32 + lane] = a;
-            continue;
-        }
-        float *o = h1s + j * kH1Stride + 4 * lane;
-        o[0] = fmaxf(fmaf(a.x, s1, bb.x), 0.f);
-        o[1] = fmaxf(fmaf(a.y, s1, bb.y), 0.f);
-        o[2] = fmaxf(fmaf(a.z, s1, bb.z), 0.f);
-        o[3] = fmaxf(fmaf(a.w, s1, bb.w), 0.f);
     }
-    if (kSplit > 1) {  // the shares of each hit, added in share order
-        __syncthreads();
-        for (int jw = warp; jw < kHitsRows; jw += kThreadsRows / 32) {
-            float4 a = part[(jw * kSplit) * 32 + lane];
+    *reinterpret_cast<float4 *>(&part[warp][4 * lane]) = a;
+    __syncthreads();
 #pragma unroll
-            for (int k = 1; k < kSplit; ++k) {
-                const float4 v = part[(jw * kSplit + k) * 32 + lane];
-                a.x += v.x;
-                a.y += v.y;
-                a.z += v.z;
-                a.w += v.w;
-            }
-            float *o = h1s + jw * kH1Stride + 4 * lane;
-            o[0] = fmaxf(fmaf(a.x, s1, bb.x), 0.f);
-            o[1] = fmaxf(fmaf(a.y, s1, bb.y), 0.f);
-            o[2] = fmaxf(fmaf(a.z, s1, bb.z), 0.f);
-            o[3] = fmaxf(fmaf(a.w, s1, bb.w), 0.f);
-        }
+    for (int e = tid; e < HITS * kN1; e += kThreadsRows) {
+        const int i = e / kN1, k = tid % kN1;
+        float s = part[i * kSplit][k];
+#pragma unroll
+        for (int q = 1; q < kSplit; ++q) s += part[i * kSplit + q][k];
+        h1[i][k] = fmaxf(fmaf(s, s1, b1), 0.f);
     }
     __syncthreads();
-    // dense-2 with every thread: output j of hit i is thread (32 i + j) mod 256's,
-    // an fmaf chain over k in order
-    for (int o = threadIdx.x; o < kHitsRows * kN2; o += kThreadsRows) {
-        const int i = o / kN2, j = o % kN2;
-        const float *h1 = h1s + i * kH1Stride;
-        float acc = b2[j];
-#pragma unroll 8
-        for (int k = 0; k < kN1; ++k) acc = fmaf(h1[k], w2[k][j], acc);
-        h2s[i * (kN2 + 1) + j] = acc;
+#pragma unroll
+    for (int i = 0; i < HITS; ++i) {
+        float acc = 0.f;
+#pragma unroll
+        for (int k = 0; k < kShare; k += 4) {
+            const float4 x = *reinterpret_cast<const float4 *>(&h1[i][kShare * warp + k]);
+            acc = fmaf(x.x, w2[k], acc);
+            acc = fmaf(x.y, w2[k + 1], acc);
+            acc = fmaf(x.z, w2[k + 2], acc);
+            acc = fmaf(x.w, w2[k + 3], acc);
+        }
+        part2[i][warp][lane] = acc;
     }
     __syncthreads();
-    if (threadIdx.x >= kHitsRows) return;
-    const int64_t h = h0 + threadIdx.x;
-    if (h >= n) return;
-    const float *h2 = h2s + threadIdx.x * (kN2 + 1);
-    float z[kNC + 1] = {cls_b[0], cls_b[1], cls_b[2], mic_b[0]};
+    const int64_t h = h0 + warp;
+    if (warp >= HITS || h >= n) return;
+    float v = b2;
 #pragma unroll
-    for (int j = 0; j < kN2; ++j) {
-        const float v = fmaxf(h2[j], 0.f);
-        const float4 wv = *reinterpret_cast<const float4 *>(&wc[j][0]);
-        z[0] = fmaf(v, wv.x, z[0]);
-        z[1] = fmaf(v, wv.y, z[1]);
-        z[2] = fmaf(v, wv.z, z[2]);
-        z[3] = fmaf(v, wv.w, z[3]);
+    for (int q = 0; q < kWarps; ++q) v += part2[warp][q][lane];
+    v = fmaxf(v, 0.f);
+    float z[kNC + 1];
+#pragma unroll
+    for (int c = 0; c <= kNC; ++c) {
+        z[c] = v * wc[c];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) z[c] += __shfl_xor_sync(0xffffffffu, z[c], o);
+        z[c] += bc[c];
     }
     const float m = fmaxf(fmaxf(z[0], z[1]), z[2]);
     const float e0 = expf(z[0] - m), e1 = expf(z[1] - m), e2 = expf(z[2] - m);
     const float sum = e0 + e1 + e2;
     float *out = out_rows.rows ? out_rows.rows + h * (int64_t)out_rows.stride : out_rows.dest[h];
-    out[0] = e0 / sum;
-    out[1] = e1 / sum;
-    out[2] = e2 / sum;
-    out[3] = 1.0f / (1.0f + expf(-z[kNC]));
-    if (debug_logits) {
-        out[4] = z[0];
-        out[5] = z[1];
-        out[6] = z[2];
-        out[7] = z[3];
-    }
+    if (lane < 4) out[lane] = lane < kNC ? (lane == 0 ? e0 : lane == 1 ? e1 : e2) / sum : 1.0f / (1.0f + expf(-z[kNC]));
+    if (debug_logits && lane < 4) out[4 + lane] = lane == 0 ? z[0] : lane == 1 ? z[1] : lane == 2 ? z[2] : z[3];
 }
 
 // The tail of the other launches: one CTA of 128 threads per 32 hits, the hits
@@ -356,13 +328,15 @@ cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, in
     const float s1 = w.fc1_scale;
     const float *b1 = w.fc1_b, *w2 = w.fc2_w, *b2 = w.fc2_b, *wc = w.cls_w, *bc = w.cls_b, *wm = w.mic_w,
                 *bm = w.mic_b;
-    if (rows > kManyRows) {
-        if (rows >= kSplitRows && n <= kSmallLaunch)  // a hit's rows over 4 warps, 2 hits per block
-            return launch_pdl(head_rows_kernel<2, 4>, dim3((n + 1) / 2), dim3(kThreadsRows), 0, s, partials, G,
-                              upt, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
-        if (n <= kSmallLaunch)  // 8 hits per block: more blocks, so more rows summed at once
-            return launch_pdl(head_rows_kernel<8>, dim3((n + 7) / 8), dim3(kThreadsRows), 0, s, partials, G, upt,
-                              n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
+    if (rows > kManyRows && n <= kSmallLaunch) {
+        if (n <= kOneHit)
+            return launch_pdl(head_rows_kernel<1>, dim3(n), dim3(kThreadsRows), 0, s, partials, G, upt, n_pad, n, s1,
+                              b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
+        if (n <= kTwoHits)
+            return launch_pdl(head_rows_kernel<2>, dim3((n + 1) / 2), dim3(kThreadsRows), 0, s, partials, G, upt, n_pad,
+                              n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
+        return launch_pdl(head_rows_kernel<4>, dim3((n + 3) / 4), dim3(kThreadsRows), 0, s, partials, G, upt, n_pad, n,
+                          s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
     }
     return launch_pdl(head_hits_kernel, dim3((n + kHeadHits - 1) / kHeadHits), dim3(kThreadsHits), 0, s, partials, G,
                       upt, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits, tile_done, status,
