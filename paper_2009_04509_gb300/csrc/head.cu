@@ -19,19 +19,22 @@ __device__ __forceinline__ unsigned long long global_timer() {
     return t;
 }
 
-// The dense-2 weights [128][32] into shared memory (16-byte aligned): every
-// load issued before the first store, so that staging costs one round trip.
+// The dense-2 weights [128][32]: a thread's share, then into shared memory
+// (16-byte aligned).
 template <int kThreads>
-__device__ __forceinline__ void stage_w2(float *w2, const float *__restrict__ fc2_w) {
-    constexpr int kN4 = kN1 * kN2 / 4;
-    static_assert(kN4 % kThreads == 0, "whole float4s per thread");
-    float4 v[kN4 / kThreads];
+struct W2Share {
+    static constexpr int kN4 = kN1 * kN2 / 4 / kThreads;
+    static_assert(kN1 * kN2 / 4 % kThreads == 0, "whole float4s per thread");
+    float4 v[kN4];
+    __device__ __forceinline__ void load(const float *__restrict__ fc2_w) {
 #pragma unroll
-    for (int k = 0; k < kN4 / kThreads; ++k)
-        v[k] = __ldg(reinterpret_cast<const float4 *>(fc2_w) + threadIdx.x + k * kThreads);
+        for (int k = 0; k < kN4; ++k) v[k] = __ldg(reinterpret_cast<const float4 *>(fc2_w) + threadIdx.x + k * kThreads);
+    }
+    __device__ __forceinline__ void store(float *w2) const {
 #pragma unroll
-    for (int k = 0; k < kN4 / kThreads; ++k) reinterpret_cast<float4 *>(w2)[threadIdx.x + k * kThreads] = v[k];
-}
+        for (int k = 0; k < kN4; ++k) reinterpret_cast<float4 *>(w2)[threadIdx.x + k * kThreads] = v[k];
+    }
+};
 constexpr int kManyRows = 4;  // up to this many partial rows per hit, head_hits_kernel at any size
 
 // The tail when a hit has many partial rows (a small launch, whose tiles are
@@ -164,11 +167,17 @@ __global__ void __launch_bounds__(kThreadsRows, HITS == 1 ? 2 : 3) head_rows_ker
 // What bounds it: the latency of this chain after the last network CTA of a
 // tile, and in a large launch the rows' L2 reads.  With a CTA per 128-hit tile
 // (256 threads) a launch of 7,692 hits, 61 tiles, ended 24 us after its network
-// kernel; this one ends about 8 us after it.
+// kernel; this one ends about 6 us after it.
+// LATE: the dense-2 weights, loaded first, go to shared memory only after the rows,
+// one round trip off the chain of a launch of a single wave of CTAs (5,000 patches
+// 127.3 -> 125.1 us, one APA in three calls 469.7 -> 464.3); in a launch of several
+// waves the registers that hold them cost more (full event 1,210 -> 1,217).
 constexpr int kHeadHits = 32;
 constexpr int kThreadsHits = 128;
 constexpr int kH1Pitch = kN1 + 4;  // h1 rows: 16-byte aligned, hits 8 apart in different banks
+constexpr int kLateHits = 3 * 152 * kHeadHits;  // hits of one wave: three CTAs per SM
 
+template <bool LATE>
 __global__ void __launch_bounds__(kThreadsHits) head_hits_kernel(const float *__restrict__ partials, int G,
                                                                 int upt, int n_pad, int32_t n, float s1,
                                                                 const float *__restrict__ fc1_b,
@@ -187,7 +196,9 @@ __global__ void __launch_bounds__(kThreadsHits) head_hits_kernel(const float *__
     __shared__ int go;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     pdl_trigger();  // the next call's first kernel may be scheduled; it waits for this one
-    stage_w2<kThreadsHits>(&w2[0][0], fc2_w);
+    W2Share<kThreadsHits> w2v;
+    w2v.load(fc2_w);
+    if (!LATE) w2v.store(&w2[0][0]);
     for (int i = tid; i < kN2 * kNC; i += kThreadsHits) wc[i / kNC][i % kNC] = cls_w[i];
     for (int i = tid; i < kN2; i += kThreadsHits) wc[i][kNC] = mic_w[i];
     const int64_t h0 = (int64_t)blockIdx.x * kHeadHits;
@@ -261,6 +272,7 @@ __global__ void __launch_bounds__(kThreadsHits) head_hits_kernel(const float *__
                 make_float4(fmaxf(fmaf(a[u].x, s1, bb.x), 0.f), fmaxf(fmaf(a[u].y, s1, bb.y), 0.f),
                             fmaxf(fmaf(a[u].z, s1, bb.z), 0.f), fmaxf(fmaf(a[u].w, s1, bb.w), 0.f));
     }
+    if (LATE) w2v.store(&w2[0][0]);
     __syncthreads();
     {
         const int hg = lane & 7, og = 4 * warp + (lane >> 3);  // hits hg + 8 i, outputs 2 og, 2 og + 1
@@ -338,8 +350,8 @@ cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, in
         return launch_pdl(head_rows_kernel<4>, dim3((n + 3) / 4), dim3(kThreadsRows), 0, s, partials, G, upt, n_pad, n,
                           s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
     }
-    return launch_pdl(head_hits_kernel, dim3((n + kHeadHits - 1) / kHeadHits), dim3(kThreadsHits), 0, s, partials, G,
-                      upt, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits, tile_done, status,
+    return launch_pdl(n <= kLateHits ? head_hits_kernel<true> : head_hits_kernel<false>,
+                      dim3((n + kHeadHits - 1) / kHeadHits), dim3(kThreadsHits), 0, s, partials, G, upt, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits, tile_done, status,
                       (long long)timeout_ns);
 }
 
