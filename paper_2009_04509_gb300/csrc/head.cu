@@ -351,8 +351,8 @@ cudaError_t launch_head(const DeviceWeights &w, const float *partials, int G, in
                           s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits);
     }
     return launch_pdl(n <= kLateHits ? head_hits_kernel<true> : head_hits_kernel<false>,
-                      dim3((n + kHeadHits - 1) / kHeadHits), dim3(kThreadsHits), 0, s, partials, G, upt, n_pad, n, s1, b1, w2, b2, wc, bc, wm, bm, out_rows, debug_logits, tile_done, status,
-                      (long long)timeout_ns);
+                      dim3((n + kHeadHits - 1) / kHeadHits), dim3(kThreadsHits), 0, s, partials, G, upt, n_pad, n, s1, b1,
+                      w2, b2, wc, bc, wm, bm, out_rows, debug_logits, tile_done, status, (long long)timeout_ns);
 }
 
 }  // namespace emtk
