@@ -103,7 +103,11 @@ constexpr int kBAccEmpty = kBAcc + 1;             // accumulator drained (4 epil
 constexpr int kBStall = kBAccEmpty + 1;
 constexpr int kBDrain = kBStall + 1;
 constexpr int kNumBarsSp = kBDrain + 1;
-constexpr int kOffTmemSlotSp = kOffBarSp + kNumBarsSp * 8;
+// partial-row staging: per epilogue warp 32 rows x 8 outputs, 16-byte halves swapped
+// in every other group of 4 rows (conflict-free 16-byte writes by row, reads by half)
+constexpr int kOffStageSp = (kOffBarSp + kNumBarsSp * 8 + 15) / 16 * 16;
+constexpr int kStageWarpSp = 32 * 8 * 4;
+constexpr int kOffTmemSlotSp = kOffStageSp + 4 * kStageWarpSp;
 constexpr int kOffAbortSp = kOffTmemSlotSp + 4;
 constexpr int kSmemBytesSp = kOffAbortSp + 4 + 1024;  // slack for 1024-byte alignment
 static_assert(kSmemBytesSp <= 232448, "shared memory budget");
@@ -505,16 +509,39 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
             const int64_t gp = 2 * u0 + pi;  // the pair's index in the launch
             const int pt = (int)(gp % kPairsPerTile);
             if (pi == np - 1 || pt % kSegPairs == kSegPairs - 1) {
-                // a segment's sums: to (first segment of this CTA in the tile) or onto
-                // this CTA's partial row of the tile
-                if (!warp_wait(bar(kBAcc), (uint32_t)segs_done & 1u, guard, lane)) break;
-                tc_fence_after();
+                // a segment's sums: to (first segment of this CTA in the tile) or onto this
+                // CTA's partial row of the tile.  32 outputs at a time, 8 of them through the
+                // staging: lane l then has half l % 2 of rows l / 2 and 16 + l / 2, so a load
+                // or store of the warp touches 16 lines instead of 32.  The old sums are read
+                // two blocks ahead, the first two under the segment's last MMAs, and the
+                // accumulator is handed back before the last block's stores.  (With a row per
+                // thread and each block's old sums read when it came, the dense-1 issuer
+                // waited 17,000 cycles every 44 pairs, a fifth of the kernel; now 11,000.  One APA
+                // 1,211 -> 1,183 us, 1,693 patches 125.1 -> 119.8.)
                 const int64_t tile = gp / kPairsPerTile;
                 const bool start = tile != last_tile;
                 last_tile = tile;
                 const int krow = cta - cta_of_unit(tile * kQuads, units, G);
-                const int64_t hit = tile * 128 + row;
-                float *dst = partials + ((int64_t)krow * n_pad + hit) * kN1;
+                const int64_t hit0 = tile * 128 + 32 * q4;
+                const int half = lane & 1, r0 = lane >> 1;
+                float *dst = partials + ((int64_t)krow * n_pad + hit0 + r0) * kN1 + 4 * half;
+                const bool in0 = hit0 + r0 < n, in1 = hit0 + r0 + 16 < n;
+                uint8_t *stage = gbase + kOffStageSp + q4 * kStageWarpSp;
+                uint8_t *st_w = stage + lane * 32, *st_r = stage + r0 * 32 + ((half ^ ((r0 >> 2) & 1)) << 4);
+                const int swap = ((lane >> 2) & 1) << 4;
+                float4 o[2][4][2];
+                auto read_old = [&](int c) {
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) {
+                        const float4 *p = reinterpret_cast<const float4 *>(dst + 32 * c + 8 * s);
+                        o[c & 1][s][0] = !start && in0 ? p[0] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                        o[c & 1][s][1] = !start && in1 ? p[16 * kN1 / 4] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    }
+                };
+                read_old(0);
+                read_old(1);
+                if (!warp_wait(bar(kBAcc), (uint32_t)segs_done & 1u, guard, lane)) break;
+                tc_fence_after();
 #pragma unroll
                 for (int c = 0; c < kN1 / 32; ++c) {
                     uint32_t r[32];
@@ -522,24 +549,31 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
                     tmem_ld16<16>(lane_tmem + kAccColSp + 32u * c + 16u, r);
                     tmem_ld_wait();
                     reg_fence(r);
-                    if (hit < n) {
-                        float4 *p4 = reinterpret_cast<float4 *>(dst + 32 * c);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            float4 v = make_float4(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]),
-                                                   __uint_as_float(r[4 * e + 2]), __uint_as_float(r[4 * e + 3]));
-                            if (!start) {
-                                const float4 o = p4[e];
-                                v = make_float4(__fadd_rn(o.x, v.x), __fadd_rn(o.y, v.y), __fadd_rn(o.z, v.z),
-                                                __fadd_rn(o.w, v.w));
-                            }
-                            p4[e] = v;
-                        }
+                    if (c == kN1 / 32 - 1) {  // the accumulator is read: the next segment may start
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar(kBAccEmpty));
                     }
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) {
+                        *reinterpret_cast<uint4 *>(st_w + swap) = make_uint4(r[8 * s], r[8 * s + 1], r[8 * s + 2], r[8 * s + 3]);
+                        *reinterpret_cast<uint4 *>(st_w + (16 - swap)) =
+                            make_uint4(r[8 * s + 4], r[8 * s + 5], r[8 * s + 6], r[8 * s + 7]);
+                        __syncwarp();
+                        const float4 v0 = *reinterpret_cast<const float4 *>(st_r);
+                        const float4 v1 = *reinterpret_cast<const float4 *>(st_r + 16 * 32);
+                        __syncwarp();
+                        float4 *p = reinterpret_cast<float4 *>(dst + 32 * c + 8 * s);
+                        const float4 &a = o[c & 1][s][0], &b = o[c & 1][s][1];
+                        if (in0)
+                            p[0] = make_float4(__fadd_rn(a.x, v0.x), __fadd_rn(a.y, v0.y), __fadd_rn(a.z, v0.z),
+                                               __fadd_rn(a.w, v0.w));
+                        if (in1)
+                            p[16 * kN1 / 4] = make_float4(__fadd_rn(b.x, v1.x), __fadd_rn(b.y, v1.y),
+                                                          __fadd_rn(b.z, v1.z), __fadd_rn(b.w, v1.w));
+                    }
+                    if (c + 2 < kN1 / 32) read_old(c + 2);
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kBAccEmpty));
                 // this CTA's last segment of the tile: its partial row is final, count it for the head
                 if (tile_done != nullptr && (pi == np - 1 || pt == kPairsPerTile - 1) && tile * 128 + 32 * q4 < n) {
                     __threadfence();
