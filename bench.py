@@ -384,11 +384,10 @@ def main():
     net_peak, net_peak_src = network_peak(args.precision, peaks)
     net_peak_sus, _ = network_peak(args.precision, peaks, sustained=True)
     union = window_union_bytes(planes)
-    if args.precision == "fp32":  # the fp32 path writes every patch
-        patch_bytes = nhits * 48 * 48 * 4
-    elif args.precision == "tf32":  # the split path writes 4-byte interval words
+    # the interval image is written; the network reads the windows from it
+    if args.precision in ("fp32", "tf32"):  # 4 bytes per interval
         patch_bytes = sum(p.nwires * (p.nticks // 6) for p in planes) * 4
-    else:  # the 16-bit paths write the interval image; the network reads the windows from it
+    else:
         patch_bytes = sum(p.nwires * (p.nticks // 6) for p in planes) * 2
     cut_ms = (kms["intervals"] + kms["gather"]) / args.steps
     cut_gbs = (union + patch_bytes) / (cut_ms / 1e3) / 1e9
@@ -430,10 +429,9 @@ def main():
         "extraction": {"bound": "hbm", "achieved": cut_gbs, "peak": peaks["hbm"], "unit": "GB/s",
                        "frac": cut_gbs / peaks["hbm"], "algorithmic_bytes": union + patch_bytes,
                        "bytes_read": union, "bytes_written": patch_bytes,
-                       "kernels": "interval_image_kernel + gather_kernel" if args.precision == "fp32" else
-                       ("mark_tiles_kernel + interval_tiles_kernel (the image tiles some window touches, and the "
-                        "window descriptors)" if tiled_cut(planes) else
-                        "interval_desc_kernel (images + window descriptors, one launch)"),
+                       "kernels": "mark_tiles_kernel + interval_tiles_kernel (the image tiles some window touches, "
+                       "and the window descriptors)" if tiled_cut(planes) and args.precision != "fp32" else
+                       "interval_desc_kernel (images + window descriptors, one launch)",
                        "ms_per_step": cut_ms},
         "step_ms_stats": {"median": statistics.median(step_ms), "min": min(step_ms), "max": max(step_ms),
                           "mean": total_ms / args.steps, "n": len(step_ms)},

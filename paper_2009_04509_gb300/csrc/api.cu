@@ -190,8 +190,8 @@ emtk_status ensure_dimg(emtk_ctx *c, size_t bytes, cudaStream_t s) {
 }
 
 // Network on `n` patches already in the workspace format -> scores via dest.
-// `desc` (tensor-core path only) locates each hit's window in the haloed
-// interval images at `patches`; without it `patches` holds the patches.
+// `desc` locates each hit's window in the haloed interval images at `patches`;
+// without it `patches`, or src32 in fp32, holds the patches.
 emtk_status run_network(emtk_ctx *c, const void *patches, const HitDesc *desc, int32_t n, OutRows out_rows,
                         const float *src32, cudaStream_t s) {
     if (n <= 0) return EMTK_OK;
@@ -213,7 +213,8 @@ emtk_status run_network(emtk_ctx *c, const void *patches, const HitDesc *desc, i
         Prof prof(c, EMTK_KERNEL_NETWORK, s);
         e = tc ? launch_cnn_tc(c->w, patches, desc, tc_mode(c->opt.precision), n, G, c->ws.partials, n_pad,
                                c->ws.status, c->opt.wait_timeout_ns, c->opt.debug_stall, tile_done, src32, s)
-               : launch_cnn_fp32(c->w, static_cast<const float *>(patches), n, G, c->ws.partials, n_pad, s);
+               : launch_cnn_fp32(c->w, src32 ? src32 : static_cast<const float *>(patches), desc, n, G, c->ws.partials,
+                                 n_pad, s);
     }
     if (e != cudaSuccess) return cuda_status(e);
     {
@@ -302,7 +303,7 @@ emtk_status run_requests(emtk_ctx *c, const emtk_request *reqs, int32_t nreq, cu
         int64_t hits;
         size_t img_bytes;
         const bool tc = tensor_precision(c->opt.precision);
-        build_table(c, reqs, r0, r1, fmt, tc ? kHalo : 0, *t, hits, img_bytes);
+        build_table(c, reqs, r0, r1, fmt, kHalo, *t, hits, img_bytes);
         if (hits == 0) continue;
         // planes of requests without hits need no interval image
         for (int i = 0; i < t->n; ++i)
@@ -323,8 +324,8 @@ emtk_status run_requests(emtk_ctx *c, const emtk_request *reqs, int32_t nreq, cu
         }
         cudaError_t e;
         {
-            // the tensor-core kernel reads the windows straight from the images; the
-            // first chunk's window descriptors are built in the same launch
+            // the network kernel reads the windows straight from the images; the first
+            // chunk's window descriptors are built in the same launch
             const DescJob job{0, (int32_t)std::min<int64_t>(c->max_hits, hits), c->ws.hdesc, c->ws.dest,
                               out_stride(c)};
             Prof prof(c, EMTK_KERNEL_INTERVALS, s, tiles ? 2 : 1);  // the tiled cut: marks, then tiles
@@ -337,7 +338,7 @@ emtk_status run_requests(emtk_ctx *c, const emtk_request *reqs, int32_t nreq, cu
                 else
                     c->tile_mask_cap = 0;  // the next call reallocates and zeroes both halves
             } else {
-                e = launch_interval_images(*t, c->ws.dimg, fmt, s, tc ? &job : nullptr);
+                e = launch_interval_images(*t, c->ws.dimg, fmt, s, &job);
             }
         }
         if (e != cudaSuccess) {
@@ -346,20 +347,16 @@ emtk_status run_requests(emtk_ctx *c, const emtk_request *reqs, int32_t nreq, cu
         }
         for (int64_t g0 = 0; g0 < hits && st == EMTK_OK; g0 += c->max_hits) {
             const int32_t cnt = (int32_t)std::min<int64_t>(c->max_hits, hits - g0);
-            if (tc && g0 > 0) {
+            if (g0 > 0) {
                 Prof prof(c, EMTK_KERNEL_GATHER, s);
                 e = launch_hit_desc(*t, g0, cnt, c->ws.hdesc, c->ws.dest, out_stride(c), s);
-            } else if (!tc) {
-                Prof prof(c, EMTK_KERNEL_GATHER, s);
-                e = launch_gather(*t, c->ws.dimg, fmt, g0, cnt, c->ws.patches, c->ws.dest, out_stride(c), s);
             }
             if (e != cudaSuccess) {
                 st = cuda_status(e);
                 break;
             }
             const OutRows out{c->ws.dest, nullptr, 0};
-            st = tc ? run_network(c, c->ws.dimg, c->ws.hdesc, cnt, out, nullptr, s)
-                    : run_network(c, c->ws.patches, nullptr, cnt, out, nullptr, s);
+            st = run_network(c, c->ws.dimg, c->ws.hdesc, cnt, out, nullptr, s);
         }
         c->stats.hits += hits;
     }
@@ -368,17 +365,16 @@ emtk_status run_requests(emtk_ctx *c, const emtk_request *reqs, int32_t nreq, cu
 }
 
 // Workspace of a context, sized by its max_hits.  The patch buffer is only
-// needed by the fp32 path and emtk_infer_patches (`patches`).
+// needed by emtk_infer_patches (`patches`).
 cudaError_t alloc_workspace(emtk_ctx *c, bool patches) {
     const emtk_options &o = c->opt;
     const emtk_patch_format fmt = patch_format(o.precision);
     cudaError_t e = cudaSuccess;
-    // the 16-bit and fp8 tensor-core kernels read pre-cut fp32 patches themselves
-    if ((patches && fmt == kPatchSplit16) || !tensor_precision(o.precision))
+    // every kernel but EMTK_TF32's reads pre-cut fp32 patches itself
+    if (patches && fmt == kPatchSplit16)
         e = dmalloc(&c->ws.patches, (size_t)o.max_hits * kPatchElems * patch_elem_bytes(fmt));
     if (e == cudaSuccess) e = dmalloc(&c->ws.dest, (size_t)o.max_hits * sizeof(float *));
-    if (e == cudaSuccess && tensor_precision(o.precision))
-        e = dmalloc(&c->ws.hdesc, (size_t)o.max_hits * sizeof(HitDesc));
+    if (e == cudaSuccess) e = dmalloc(&c->ws.hdesc, (size_t)o.max_hits * sizeof(HitDesc));
     if (e == cudaSuccess) {
         c->ws.partial_elems = (size_t)std::max<int64_t>(kPartialCap, (int64_t)n_pad_of(o.max_hits) * kN1);
         e = dmalloc(&c->ws.partials, c->ws.partial_elems * sizeof(float));
@@ -578,7 +574,7 @@ emtk_status emtk_extract_patches(emtk_ctx *c, const float *d_adc, int32_t nwires
     }
     if (st == EMTK_OK) {
         Prof prof(c, EMTK_KERNEL_GATHER, s);
-        st = cuda_status(launch_gather(*t, c->ws.dimg, fmt, 0, nhits, d_patches, nullptr, 0, s));
+        st = cuda_status(launch_gather(*t, c->ws.dimg, fmt, nhits, d_patches, s));
     }
     c->stats.calls++;
     delete t;
@@ -601,10 +597,7 @@ emtk_status emtk_infer_patches(emtk_ctx *c, const float *d_patches, int32_t n, f
         const float *src = d_patches + h0 * kPatchElems;
         // the head writes hit h's scores to rows + h * stride (no pointer table)
         const OutRows out{nullptr, d_scores + h0 * out_stride(c), out_stride(c)};
-        if (fmt == EMTK_PATCH_BF16 || fmt == EMTK_PATCH_F16) {
-            // the tensor-core kernel reads the fp32 patches itself: no conversion launch
-            st = run_network(c, nullptr, nullptr, cnt, out, src, s);
-        } else if (fmt == kPatchSplit16) {
+        if (fmt == kPatchSplit16) {
             {
                 // the split-fp16 network reads head / tail words: one conversion launch first
                 Prof prof(c, EMTK_KERNEL_CONVERT, s);
@@ -612,7 +605,8 @@ emtk_status emtk_infer_patches(emtk_ctx *c, const float *d_patches, int32_t n, f
             }
             if (st == EMTK_OK) st = run_network(c, c->ws.patches, nullptr, cnt, out, nullptr, s);
         } else {
-            st = run_network(c, src, nullptr, cnt, out, nullptr, s);  // the fp32 kernel reads the patches
+            // the other kernels read the fp32 patches themselves: no conversion launch
+            st = run_network(c, nullptr, nullptr, cnt, out, src, s);
         }
     }
     c->stats.calls++;

@@ -149,9 +149,26 @@ __device__ __forceinline__ void fma_frag(const Frag &f, float2 (&acc)[8][8]) {
     }
 }
 
-// units = tiles * kPairs pairs in all; seg: positions per dense-1 segment.
+// Eight pixels of a window row whose first is element m (0..3) of the aligned
+// 16-byte chunk at p; the third chunk is read only if it is needed.
+__device__ __forceinline__ void load_pixels8(const float4 *__restrict__ p, int m, float4 &lo, float4 &hi) {
+    const float4 a = __ldg(p), b = __ldg(p + 1), c = m ? __ldg(p + 2) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float w[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
+    float s[10], o[8];
+#pragma unroll
+    for (int j = 0; j < 10; ++j) s[j] = (m & 2) ? w[j + 2] : w[j];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) o[j] = (m & 1) ? s[j + 1] : s[j];
+    lo = make_float4(o[0], o[1], o[2], o[3]);
+    hi = make_float4(o[4], o[5], o[6], o[7]);
+}
+
+// units = tiles * kPairs pairs in all; seg: positions per dense-1 segment.  src:
+// patches [n][48][48] (desc null), or the haloed interval images of the hits'
+// planes, located through desc.
 __global__ void __launch_bounds__(kThreads, 1)
-    cnn_fp32_kernel(const float *__restrict__ patches, int n, const float *__restrict__ conv_w,
+    cnn_fp32_kernel(const float *__restrict__ src, const HitDesc *__restrict__ desc, int n,
+                    const float *__restrict__ conv_w,
                     const float *__restrict__ conv_b, const float *__restrict__ fc1_w, long long units,
                     float *__restrict__ partials, int n_pad, int seg) {
     extern __shared__ float4 smem_f4[];
@@ -174,19 +191,47 @@ __global__ void __launch_bounds__(kThreads, 1)
             load_w1(w1, fc1_w, p, t);
             load_w1(w1 + kW1Pos, fc1_w, p + 1, t);
         }
-        pdl_wait();  // the patches come from the kernel before
+        pdl_wait();  // the patches, or images and descriptors, come from the kernel before
+        HitDesc hd;  // of hit t of the tile
+        bool have = false;
         const int hit_c = 64 * ((t >> 5) & 1) + (t & 31), f_c = 24 * (t >> 6);  // this thread's conv: hits, filters
         for (int i = 0; i < np; i += 2) {
             // the pair of position p: window rows y .. y+4, columns x0 .. x0+7 of its quad
             const int y = p / kQ, x = p - y * kQ, x0 = x & ~3;
             if (i == 0 || x == x0) {  // a new quad: thread t stages hit t's window
                 const int64_t hit = tile * kHT + t;
-                const float4 *src = reinterpret_cast<const float4 *>(patches + hit * kPatchElems + y * kPatch + x0);
+                if (!have) {
+                    have = true;
+                    if (desc != nullptr && hit < n) {
+                        hd = desc[hit];
+                    } else {
+                        hd.origin = hit < n ? hit * kPatchElems : 0;
+                        hd.pitch = kPatch;
+                        hd.inside = 1;
+                    }
+                }
                 float4 a[kK], b[kK];
+                if (hit < n && hd.inside) {  // the pitch is a multiple of 4: every row has the phase m
+                    const int m = (int)(hd.origin & 3);
+                    const float *p = src + (hd.origin - m) + (int64_t)y * hd.pitch + x0;
 #pragma unroll
-                for (int r = 0; r < kK; ++r) {
-                    a[r] = hit < n ? __ldg(src + r * (kPatch / 4)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                    b[r] = hit < n ? __ldg(src + r * (kPatch / 4) + 1) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    for (int r = 0; r < kK; ++r)
+                        load_pixels8(reinterpret_cast<const float4 *>(p + (int64_t)r * hd.pitch), m, a[r], b[r]);
+                } else {  // past the last hit, or a hit outside its plane: every pixel checked
+#pragma unroll
+                    for (int r = 0; r < kK; ++r) {
+                        float v[8];
+                        const int w = hd.wc - kHalf + y + r;
+                        const bool wok = hit < n && w >= 0 && w < hd.nwires;
+                        const float *row = src + (wok ? hd.d_off + (int64_t)(w + kHalo) * hd.pitch + kHalo : 0);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const int64_t c = (int64_t)hd.bc - kHalf + x0 + j;
+                            v[j] = wok && c >= 0 && c < hd.nint ? __ldg(row + c) : 0.0f;
+                        }
+                        a[r] = make_float4(v[0], v[1], v[2], v[3]);
+                        b[r] = make_float4(v[4], v[5], v[6], v[7]);
+                    }
                 }
                 bar_conv();  // the last quad's window has been read (first: the conv weights are staged)
 #pragma unroll
@@ -213,6 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (p == kPos) {
                 p = 0;
                 ++tile;
+                have = false;
             }
         }
         return;
@@ -295,13 +341,13 @@ cudaError_t init_fp32_kernel_attrs() {
     return cudaFuncSetAttribute(cnn_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
 }
 
-cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *patches, int32_t n, int G, float *partials,
-                            int n_pad, cudaStream_t s) {
+cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *src, const HitDesc *desc, int32_t n, int G,
+                            float *partials, int n_pad, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const long long units = (long long)((n + kHT - 1) / kHT) * kPairs;
     const int seg = units <= 88ll * G ? 16 : kQ;
     const float *cw = w.conv_w, *cb = w.conv_b, *fw = w.fc1_w;
-    return launch_pdl(cnn_fp32_kernel, dim3(G), dim3(kThreads), kSmemBytes, s, patches, n, cw, cb, fw, units,
+    return launch_pdl(cnn_fp32_kernel, dim3(G), dim3(kThreads), kSmemBytes, s, src, desc, n, cw, cb, fw, units,
                       partials, n_pad, seg);
 }
 

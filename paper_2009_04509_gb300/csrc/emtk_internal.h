@@ -118,8 +118,8 @@ struct HfTable {
 struct Workspace {
     void *dimg = nullptr;        // interval images of the planes of one launch
     size_t dimg_bytes = 0;
-    void *patches = nullptr;     // [max_hits][48][48] in the precision's patch format
-    HitDesc *hdesc = nullptr;    // [max_hits] window descriptors (tensor-core path)
+    void *patches = nullptr;     // [max_hits][48][48] split-fp16 words (EMTK_TF32, emtk_infer_patches)
+    HitDesc *hdesc = nullptr;    // [max_hits] window descriptors
     float **dest = nullptr;      // [max_hits] output row of each hit
     float *partials = nullptr;   // [rows][n_pad][128] of the running launch
     size_t partial_elems = 0;
@@ -284,10 +284,9 @@ cudaError_t launch_interval_images(const ReqTable &t, void *dimg, emtk_patch_for
 cudaError_t launch_cut_tiles(const ReqTable &t, int64_t total_hits, void *dimg, emtk_patch_format fmt,
                              const DescJob &job, uint32_t *mask_cur, uint32_t *mask_next, int64_t mask_cap,
                              cudaStream_t s);
-// Patches of hits [g0, g0+count) of the concatenated list (global index).
-// Writes patches[(g - g0)] and, if dest != null, dest[g - g0] = output row.
-cudaError_t launch_gather(const ReqTable &t, const void *dimg, emtk_patch_format fmt, int64_t g0,
-                          int32_t count, void *patches, float **dest, int out_stride, cudaStream_t s);
+// Patches of the first `count` hits of the concatenated list.
+cudaError_t launch_gather(const ReqTable &t, const void *dimg, emtk_patch_format fmt, int32_t count, void *patches,
+                          cudaStream_t s);
 // Pre-cut fp32 patches (n values, a multiple of 8, 16-byte aligned) into the
 // split-fp16 head / tail words of the EMTK_TF32 network at dst (n words), in
 // one launch of at most 8 CTAs per SM.
@@ -307,10 +306,10 @@ int64_t find_hits_chunks(const HfTable &t, int64_t nunits);
 cudaError_t launch_find_hits(const HfTable &t, int64_t nunits, void *scratch, int32_t *sums_cur, int32_t *sums_next,
                              int64_t cap, int32_t *totals, cudaStream_t s);
 
-// Network in fp32: dense-1 partial sums [rows][n_pad][128] from patches, stream-K
-// over G CTAs in pairs of positions (rows = streamk_partial_rows(n, G, kPos / 2)).
-cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *patches, int32_t n, int G, float *partials,
-                            int n_pad, cudaStream_t s);
+// Network in fp32: dense-1 partial sums [rows][n_pad][128] from patches (desc
+// null) or from the hits' windows in the haloed interval images, stream-K over G CTAs in pairs of positions (rows = streamk_partial_rows(n, G, kPos / 2)).
+cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *src, const HitDesc *desc, int32_t n, int G,
+                            float *partials, int n_pad, cudaStream_t s);
 // Stream-K over G CTAs (one per SM); partials [rows][n_pad][128] with rows
 // = streamk_partial_rows(n, G, kQuads).
 // src: 16-bit patches [n][48][48] (desc == nullptr) or the haloed interval

@@ -203,24 +203,19 @@ __device__ __forceinline__ uint4 shift_chunk(const uint4 &lo, const uint4 &hi, i
 
 template <int FMT>
 __global__ void __launch_bounds__(kGatherThreads) gather_kernel(const __grid_constant__ ReqTable t, const void *img,
-                                                                int64_t g0, void *patches, float **dest,
-                                                                int out_stride) {
+                                                                void *patches) {
     using G = Gather<FMT>;
     using T = typename G::T;
     pdl_trigger();  // the next kernel may set up while this one runs; it waits for it
-    const int64_t local = blockIdx.x;
-    const int64_t g = g0 + local;
-    const int ri = find_request(t, g);
-    const ReqDesc &r = t.r[ri];
-    const int64_t hloc = g - r.hit_begin;
+    const int64_t g = blockIdx.x;
+    const ReqDesc &r = t.r[find_request(t, g)];
     if (r.nwires == 0) pdl_wait();  // no image kernel may stand between this one and what wrote the hits
-    const emtk_hit hit = r.hits[hloc];
+    const emtk_hit hit = r.hits[g - r.hit_begin];
     const int64_t wc = hit.wire;
     const int64_t bc = floor_div6(hit.tick);
-    T *out = static_cast<T *>(patches) + local * kPatchElems;
+    T *out = static_cast<T *>(patches) + g * kPatchElems;
     const int c = threadIdx.x % G::CH, row0 = threadIdx.x / G::CH;
     pdl_wait();  // the images come from the kernel before
-    if (dest != nullptr && threadIdx.x == 0) dest[local] = r.scores + hloc * out_stride;
     const T *src = static_cast<const T *>(img) + r.d_off;
     const int64_t w0 = wc - kHalf + r.halo, b0 = bc - kHalf + r.halo;  // the window's first image row, column
     if (r.nwires > 0 && w0 >= 0 && w0 + kPatch <= r.nwires + 2 * (int64_t)r.halo && b0 >= 0 &&
@@ -570,14 +565,13 @@ cudaError_t launch_cut_tiles(const ReqTable &t, int64_t total_hits, void *dimg, 
                       mask_next, mask_cap, job.g0, job.count, job.desc, job.dest, job.out_stride);
 }
 
-cudaError_t launch_gather(const ReqTable &t, const void *dimg, emtk_patch_format fmt, int64_t g0, int32_t count,
-                          void *patches, float **dest, int out_stride, cudaStream_t s) {
+cudaError_t launch_gather(const ReqTable &t, const void *dimg, emtk_patch_format fmt, int32_t count, void *patches,
+                          cudaStream_t s) {
     if (count <= 0) return cudaSuccess;
     auto *kernel = fmt == EMTK_PATCH_F32    ? gather_kernel<EMTK_PATCH_F32>
                    : fmt == EMTK_PATCH_BF16 ? gather_kernel<EMTK_PATCH_BF16>
                                             : gather_kernel<EMTK_PATCH_F16>;
-    return launch_pdl(kernel, dim3((unsigned)count), dim3(kGatherThreads), 0, s, t, dimg, g0, patches, dest,
-                      out_stride);
+    return launch_pdl(kernel, dim3((unsigned)count), dim3(kGatherThreads), 0, s, t, dimg, patches);
 }
 
 cudaError_t launch_convert_split(const float *src, void *dst, int64_t n, int sms, cudaStream_t s) {
