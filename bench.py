@@ -1,7 +1,7 @@
 """Benchmark: EmTrackMichelId hit identification on GB300.
 
 One step = one pass of the whole hot path over one synthetic event: the
-patch cut (time-interval image + gather), the fused conv + dense-1 tensor-core
+patch cut (time-interval images), the fused conv + dense-1 tensor-core
 kernel and the dense-2/heads kernel, for all 18 planes of a full 6-APA event
 (15,360 wires x 6000 ticks, 60,000 hits) in one batched call
 (emtk_infer_batch), bf16.  Inputs are device-resident when a timed step
@@ -37,9 +37,9 @@ METRIC = "hit patches/sec on 1 GB300 (extract+CNN); % bf16 tensor peak; gather H
 # precision, each from one ncu capture of this benchmark (profiles/launch_list_full_event_*.md),
 # with the kernel source it was taken on: reported as null once that source changes.
 TC_TRAFFIC = {
-    "bf16": (51_517_440 + 9_344_512, "cnn_tc.cu", "d9c50f1f72130cf7"),
-    "fp8": (38_985_728 + 3_194_880, "cnn_tc.cu", "d9c50f1f72130cf7"),
-    "tf32": (979_775_744 + 435_545_600, "cnn_split.cu", "b3b11cc28934b03a"),
+    "bf16": (51_453_184 + 9_233_408, "cnn_tc.cu", "34292476b30d1965"),
+    "fp8": (38_927_104 + 3_178_752, "cnn_tc.cu", "34292476b30d1965"),
+    "tf32": (1_143_539_200 + 455_674_112, "cnn_split.cu", "98a464f94542f84c"),
 }
 
 
@@ -655,8 +655,8 @@ def run_sweep(args, rank, world, local_rank):
 HITFIND_THRESHOLD = 15.0  # 5 sigma of the synthetic planes' noise
 # DRAM bytes (read + write) of one hf_find_kernel launch on the full event, from one ncu
 # capture of this workload (profiles/hitfind_full_event.md); null once hitfind.cu changes.
-HF_TRAFFIC_BYTES = 369_188_864 + 4_362_496
-HF_TRAFFIC_SOURCE_SHA256 = "2ba949573c38cacd"
+HF_TRAFFIC_BYTES = 369_231_872 + 4_092_416
+HF_TRAFFIC_SOURCE_SHA256 = "3cf4d6e9c5e60e51"
 
 
 def hf_traffic():

@@ -146,7 +146,7 @@ typedef struct {
 /* Kernel classes of the hot path, for per-kernel timing. */
 typedef enum {
     EMTK_KERNEL_INTERVALS = 0, /* plane -> time-interval image */
-    EMTK_KERNEL_GATHER = 1,    /* interval image -> 48x48 patches */
+    EMTK_KERNEL_GATHER = 1,    /* interval image -> 48x48 patches, later chunks' window descriptors */
     EMTK_KERNEL_NETWORK = 2,   /* conv + dense-1 (tensor cores or fp32) */
     EMTK_KERNEL_HEAD = 3,      /* dense-1 sum + dense-2 + heads */
     EMTK_KERNEL_CONVERT = 4,   /* fp32 patches -> split-fp16 words (emtk_infer_patches, EMTK_TF32) */

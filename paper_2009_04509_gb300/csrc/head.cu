@@ -5,7 +5,7 @@
 // from the stream-K CTAs that shared its tile.
 // Two kernels, chosen by launch_head, each with its sums in a fixed order:
 //   head_rows_kernel  small launches, whose tiles are spread over many CTAs: a
-//                     CTA per hit or two, its warps share the hit's many rows;
+//                     CTA per one, two or four hits, its warps share the hit's many rows;
 //   head_hits_kernel  the others: a CTA per 32 hits, the share of one epilogue
 //                     warp of the network kernels.
 #include "emtk_internal.h"
