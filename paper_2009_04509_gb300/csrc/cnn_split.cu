@@ -477,6 +477,9 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
         const uint32_t lane_tmem = tmem + ((uint32_t)(32 * q4) << 16);
         int segs_done = 0;
         int64_t last_tile = -1;  // tile whose partial row this CTA has started
+        // partial row of the CTA's first tile (of the others, which begin in its range, row
+        // 0): its 64-bit divisions are not left to the drains
+        const int krow0 = cta - cta_of_unit((int64_t)tile0 * kQuads, units, G);
         for (int pi = 0; pi < np; ++pi) {
             const int s = pi % kSlotsSp;
             if (!warp_wait(bar(kBConv + s), (uint32_t)(pi / kSlotsSp) & 1u, guard, lane)) break;
@@ -521,7 +524,7 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
                 const int64_t tile = gp / kPairsPerTile;
                 const bool start = tile != last_tile;
                 last_tile = tile;
-                const int krow = cta - cta_of_unit(tile * kQuads, units, G);
+                const int krow = tile == tile0 ? krow0 : 0;
                 const int64_t hit0 = tile * 128 + 32 * q4;
                 const int half = lane & 1, r0 = lane >> 1;
                 float *dst = partials + ((int64_t)krow * n_pad + hit0 + r0) * kN1 + 4 * half;
