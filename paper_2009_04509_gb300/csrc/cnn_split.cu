@@ -85,6 +85,14 @@ constexpr float kActScaleSp = 0.0625f;                        // s_a
 // (792 MMAs) and the epilogue adds each segment's sums to the CTA's partial
 // row with round-to-nearest fp32 adds, in pair order (deterministic).
 constexpr int kSegPairs = 44;
+// Pairs the epilogue converts between the end of a segment and its drain: the
+// dense-1 issuer's work from the moment it has the accumulator back.  A pair of
+// the next segment needs the slot of the pair four before it, so up to three
+// can be converted before that segment's own MMAs start.  Measured with 0, 1, 2:
+// one APA 1,166, 1,152, 1,160 us, 1,693 patches 117.7, 116.7, 118.0, 300 patches
+// 43.2, 42.3, 42.4 (later, the wait for the sums is over before the old sums are in).
+constexpr int kDefer = 1;
+static_assert(kDefer < kSlotsSp && kDefer < kSegPairs, "the pairs converted before a drain need no MMA after it");
 static_assert((2 * kQuads) % kSegPairs == 0, "segments tile the pairs of a tile");
 
 constexpr int kOffW1Sp = 0;
@@ -477,6 +485,7 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
         const uint32_t lane_tmem = tmem + ((uint32_t)(32 * q4) << 16);
         int segs_done = 0;
         int64_t last_tile = -1;  // tile whose partial row this CTA has started
+        int pend = -1;           // last pair of the segment to be drained
         // partial row of the CTA's first tile (of the others, which begin in its range, row
         // 0): its 64-bit divisions are not left to the drains
         const int krow0 = cta - cta_of_unit((int64_t)tile0 * kQuads, units, G);
@@ -509,9 +518,14 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBAct + s));
-            const int64_t gp = 2 * u0 + pi;  // the pair's index in the launch
-            const int pt = (int)(gp % kPairsPerTile);
-            if (pi == np - 1 || pt % kSegPairs == kSegPairs - 1) {
+            // The segment that ended kDefer pairs ago is drained now (at the CTA's last pair
+            // what is left of both).
+            const bool end = pi == np - 1 || (int)((2 * u0 + pi) % kPairsPerTile) % kSegPairs == kSegPairs - 1;
+            if (end && pend < 0) pend = pi;
+            bool gave_up = false;
+            while (pend >= 0 && (pi == np - 1 || pi >= pend + kDefer)) {
+                const int64_t gp = 2 * u0 + pend;  // the segment's last pair, its index in the launch
+                const int pt = (int)(gp % kPairsPerTile);
                 // a segment's sums: to (first segment of this CTA in the tile) or onto this
                 // CTA's partial row of the tile.  32 outputs at a time, 8 of them through the
                 // staging: lane l then has half l % 2 of rows l / 2 and 16 + l / 2, so a load
@@ -519,8 +533,9 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
                 // two blocks ahead, the first two under the segment's last MMAs, and the
                 // accumulator is handed back before the last block's stores.  (With a row per
                 // thread and each block's old sums read when it came, the dense-1 issuer
-                // waited 17,000 cycles every 44 pairs, a fifth of the kernel; now 11,000.  One APA
-                // 1,211 -> 1,183 us, 1,693 patches 125.1 -> 119.8.)
+                // waited 17,000 cycles every 44 pairs, a fifth of the kernel; then 11,000, and with
+                // a pair converted ahead (kDefer) 9,000.  One APA 1,211 -> 1,183 -> 1,152 us, 1,693
+                // patches 125.1 -> 118.3 -> 116.7.)
                 const int64_t tile = gp / kPairsPerTile;
                 const bool start = tile != last_tile;
                 last_tile = tile;
@@ -543,7 +558,10 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
                 };
                 read_old(0);
                 read_old(1);
-                if (!warp_wait(bar(kBAcc), (uint32_t)segs_done & 1u, guard, lane)) break;
+                if (!warp_wait(bar(kBAcc), (uint32_t)segs_done & 1u, guard, lane)) {
+                    gave_up = true;
+                    break;
+                }
                 tc_fence_after();
 #pragma unroll
                 for (int c = 0; c < kN1 / 32; ++c) {
@@ -578,13 +596,15 @@ __global__ void __launch_bounds__(kThreadsSp, 1)
                     if (c + 2 < kN1 / 32) read_old(c + 2);
                 }
                 // this CTA's last segment of the tile: its partial row is final, count it for the head
-                if (tile_done != nullptr && (pi == np - 1 || pt == kPairsPerTile - 1) && tile * 128 + 32 * q4 < n) {
+                if (tile_done != nullptr && (pend == np - 1 || pt == kPairsPerTile - 1) && tile * 128 + 32 * q4 < n) {
                     __threadfence();
                     __syncwarp();
                     if (lane == 0) atomicAdd(tile_done + 4 * tile + q4, 1);
                 }
                 ++segs_done;
+                pend = end && pend != pi ? pi : -1;
             }
+            if (gave_up) break;
         }
     }
 
