@@ -24,14 +24,17 @@
 // fully unrolled conv took 6,000 cycles per position for 1,200 FMAs).
 //
 // What bounds it: the FMA pipe.  A position is 7,344 pipe cycles; it takes about
-// 9,300 (20,096 hits: 9.6 ms, 60 TFLOP/s, 0.75 of the derived peak; the kernel
-// before this one 13.5 ms).  Operands that are all 64-bit pairs straight from
+// 9,400 (one APA, 20,000 hits: 9.3 ms, 61 TFLOP/s, 0.75 of the derived peak; the
+// kernel before this one 13.6 ms).  Operands that are all 64-bit pairs straight from
 // shared memory (each activation stored twice, no copies) ran at 42 TFLOP/s, an
 // 8 x 8 register tile on twice the warps at 59, scalar FMAs at 53.
 //
-// The dense-1 sums restart every `seg` positions of a tile and are added to
+// The dense-1 sums restart every kSeg positions of a tile and are added to
 // the CTA's partial row of the tile with one fp32 add per segment, in order
-// (deterministic; shorter chains of sums round less).  The head kernel adds
+// (deterministic; shorter chains of sums round less: scores of 2,080 patches
+// are off by 9.8e-7 against 64 bits with 16 positions, 1.4e-6 with 44, 8.0e-7
+// with 8, and 1.7e-6 in the kernel before this one; with 44 the kernel is 1.2 %
+// faster, with 8 3 % slower).  The head kernel adds
 // the partial rows of the CTAs that shared a tile, in CTA order.
 #include "emtk_internal.h"
 
@@ -43,6 +46,7 @@ constexpr int kRole = 128;        // threads of each role
 constexpr int kThreads = 2 * kRole;
 constexpr int kPairs = kPos / 2;   // units per tile: pairs of conv positions (x, x + 1), x even
 constexpr int kSlots = 4;          // ring slots (positions)
+constexpr int kSeg = 16;           // positions per dense-1 segment
 constexpr int kW1Pos = kF * kN1;   // 6144 weights of one position (24 KB)
 constexpr int kActPos = kF * kHT;  // 6144 activations of one position
 constexpr int kWinHalf = kK * kHT * 4;      // 5 rows x 128 hits x 4 columns of a quad's window
@@ -163,14 +167,13 @@ __device__ __forceinline__ void load_pixels8(const float4 *__restrict__ p, int m
     hi = make_float4(o[4], o[5], o[6], o[7]);
 }
 
-// units = tiles * kPairs pairs in all; seg: positions per dense-1 segment.  src:
-// patches [n][48][48] (desc null), or the haloed interval images of the hits'
-// planes, located through desc.
+// units = tiles * kPairs pairs in all.  src: patches [n][48][48] (desc null), or
+// the haloed interval images of the hits' planes, located through desc.
 __global__ void __launch_bounds__(kThreads, 1)
     cnn_fp32_kernel(const float *__restrict__ src, const HitDesc *__restrict__ desc, int n,
                     const float *__restrict__ conv_w,
                     const float *__restrict__ conv_b, const float *__restrict__ fc1_w, long long units,
-                    float *__restrict__ partials, int n_pad, int seg) {
+                    float *__restrict__ partials, int n_pad) {
     extern __shared__ float4 smem_f4[];
     float *w1 = reinterpret_cast<float *>(smem_f4);  // [kSlots][48][128]
     float *act = w1 + kSlots * kW1Pos;               // [kSlots][48][128]
@@ -278,6 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int o = 0; o < 8; ++o) acc[q][o] = make_float2(0.0f, 0.0f);
     int64_t started = -1;  // tile whose partial row this CTA has begun
+    int krow = 0;          // which of the tile's partial rows it is
     for (int i = 0; i < np; i += 2) {
         const int s = i & (kSlots - 1), b = s >> 1;
         bar_wait(kBarFull + b);
@@ -296,9 +300,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (i + kSlots < np) bar_arrive(kBarFree + b);
         p += 2;
-        if (i == np - 2 || p == kPos || p % seg == 0) {  // the segment's sums onto the partial row
-            const int krow = cta - cta_of_unit(tile * kPairs, units, G);
+        if (i == np - 2 || p == kPos || p % kSeg == 0) {  // the segment's sums onto the partial row
             const bool first = tile != started;
+            if (first) krow = cta - cta_of_unit(tile * kPairs, units, G);
             started = tile;
             // rows past n lie in the padding of the tile and are never read.  Four hits at
             // a time: their loads before their stores
@@ -345,10 +349,9 @@ cudaError_t launch_cnn_fp32(const DeviceWeights &w, const float *src, const HitD
                             float *partials, int n_pad, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const long long units = (long long)((n + kHT - 1) / kHT) * kPairs;
-    const int seg = units <= 88ll * G ? 16 : kQ;
     const float *cw = w.conv_w, *cb = w.conv_b, *fw = w.fc1_w;
     return launch_pdl(cnn_fp32_kernel, dim3(G), dim3(kThreads), kSmemBytes, s, src, desc, n, cw, cb, fw, units,
-                      partials, n_pad, seg);
+                      partials, n_pad);
 }
 
 }  // namespace emtk

@@ -1,6 +1,6 @@
 """The fp32 network kernel where its split of the work changes: one hit, the
-128-hit tile's edge, and both sides of the hit count (13.8 tiles on 152 SMs) from
-which its dense-1 segments grow from 16 to 44 positions.  Bar: the fp32 path's,
+128-hit tile's edge, and launches in which a CTA has less than one tile or more
+(13.8 tiles are 88 pairs per CTA on 152 SMs).  Bar: the fp32 path's,
 max |score difference| <= 1e-3 against the fp64 oracle."""
 import numpy as np
 import pytest
