@@ -37,9 +37,9 @@ METRIC = "hit patches/sec on 1 GB300 (extract+CNN); % bf16 tensor peak; gather H
 # precision, each from one ncu capture of this benchmark (profiles/launch_list_full_event_*.md),
 # with the kernel source it was taken on: reported as null once that source changes.
 TC_TRAFFIC = {
-    "bf16": (51_453_184 + 9_233_408, "cnn_tc.cu", "34292476b30d1965"),
-    "fp8": (38_927_104 + 3_178_752, "cnn_tc.cu", "34292476b30d1965"),
-    "tf32": (1_143_539_200 + 455_674_112, "cnn_split.cu", "98a464f94542f84c"),
+    "bf16": (51_542_016 + 9_414_144, "cnn_tc.cu", "ff64cfec79d480d2"),
+    "fp8": (38_926_080 + 3_245_056, "cnn_tc.cu", "ff64cfec79d480d2"),
+    "tf32": (1_138_716_928 + 454_535_424, "cnn_split.cu", "dd860b7b7cf67294"),
 }
 
 
